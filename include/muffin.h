@@ -161,8 +161,9 @@ int muffin_tiling(const muffin_ctx* ctx, int* fine_levels, int* cluster);
 
 /* Threads per block of the vectorised wavelet kernels of the split in use
  * (256 or 512; each block size has its own work runs per thread), chosen by
- * the set-up autotuner with the split when fine_levels < 0.  Either pointer
- * may be NULL. */
+ * the set-up autotuner with the split when fine_levels < 0.  (The fine levels
+ * of large cubes, N >= 128, march down the rows in blocks of N / 4 threads
+ * instead of these halo tiles.)  Either pointer may be NULL. */
 int muffin_block_threads(const muffin_ctx* ctx, int* fine_threads, int* coarse_threads);
 
 const char* muffin_last_error(const muffin_ctx* ctx);  /* ctx may be NULL (init errors) */

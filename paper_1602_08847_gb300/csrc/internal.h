@@ -90,6 +90,13 @@ cudaError_t launch_fine_adjoint_vec(const Geom& g, const IuwtArgs& a, cudaStream
 cudaError_t launch_coarse_vec(const Geom& g, const float* c_in, float* r_out, float* U, float k, float rho,
                               cudaStream_t s);
 cudaError_t iuwt_vec_configure();
+// The same fine levels as a march down whole-width strips (k_iuwt_march.cu),
+// and whether a cube is large enough for it.
+bool iuwt_march_analysis(const Geom& g);
+bool iuwt_march_adjoint(const Geom& g);
+cudaError_t launch_fine_analysis_march(const Geom& g, const IuwtArgs& a, cudaStream_t s);
+cudaError_t launch_fine_adjoint_march(const Geom& g, const IuwtArgs& a, cudaStream_t s);
+cudaError_t iuwt_march_configure(const Geom& g);
 cudaError_t fft_configure(int n);
 
 // ---- W_s as a union of eight orthonormal Daubechies bases (k_dwt.cu) ----

@@ -889,6 +889,7 @@ cudaError_t launch_fine_analysis(const Geom& g, const IuwtArgs& a, int mode, cud
     return cudaGetLastError();
   }
   if (nblocks) *nblocks = (g.n / kTile) * (g.n / kTile) * g.L;
+  if (mode == MODE_UPDATE && iuwt_march_analysis(g)) return launch_fine_analysis_march(g, a, s);
   if (g.vec && mode == MODE_UPDATE && iuwt_vec_fine_ok(g)) return launch_fine_analysis_vec(g, a, s);
   switch (g.gen * 10 + g.j1) {
     case 11: return fine_an_mode<1, 1>(g, a, mode, s);
@@ -918,6 +919,7 @@ template <int GEN, int J1> static cudaError_t fine_adj(const Geom& g, const Iuwt
 }
 
 cudaError_t launch_fine_adjoint(const Geom& g, const IuwtArgs& a, cudaStream_t s) {
+  if (iuwt_march_adjoint(g)) return launch_fine_adjoint_march(g, a, s);
   if (g.vec && iuwt_vec_fine_ok(g)) return launch_fine_adjoint_vec(g, a, s);
   switch (g.gen * 10 + g.j1) {
     case 11: return fine_adj<1, 1>(g, a, s);
@@ -1063,7 +1065,8 @@ cudaError_t iuwt_configure(Geom& g) {
   if (const char* v = getenv("MUFFIN_FINE_THREADS")) g.fnt = atoi(v) == 512 ? 512 : 256;
   if (const char* v = getenv("MUFFIN_COARSE_THREADS")) g.cnt = atoi(v) == 512 ? 512 : 256;
   if (g.vec) {
-    const cudaError_t e = iuwt_vec_configure();
+    cudaError_t e = iuwt_vec_configure();
+    if (e == cudaSuccess) e = iuwt_march_configure(g);
     if (e != cudaSuccess) return e;
   }
   return g.gen == 1 ? cfg_gen<1>(g) : cfg_gen<2>(g);

@@ -499,6 +499,7 @@ static int autotune_split(muffin_ctx* ctx) {
   if (any && best_g.vec && getenv("MUFFIN_FINE_THREADS") == nullptr && getenv("MUFFIN_COARSE_THREADS") == nullptr) {
     for (int fnt : {256, 512}) {
       for (int cnt : {256, 512}) {
+        if (fnt != best_g.fnt && iuwt_march_analysis(best_g)) continue;   // no halo tile left to shape
         if (fnt == best_g.fnt && cnt == best_g.cnt) continue;
         Geom g = best_g;
         g.fnt = fnt;
