@@ -181,47 +181,55 @@ struct LastArgs {
   float* out_aux;             // EPI_PRED: fields [nz][K-1][ny][nx]
 };
 
-// ------------------------------------------------------------------ 32 -> 32 layers on tcgen05 (UMMA), fed by TMA
+// ------------------------------------------------------------------ 32 -> 32 layers on tcgen05 (UMMA), marching along z
 //
-// One CTA of 128 threads walks output tiles of 128 voxels (one channel, 16
-// rows, 8 columns).  For each tile D[128 voxels][32 features] accumulates in
-// tensor memory over 27 taps x 2 steps of K = 16 by tcgen05.mma (kind::f16,
-// bfloat16 A and B, float32 D, M = 128, N = 32; N = 16 for the last layer,
-// whose epilogue writes the prediction or the loss terms); both operands are read from
-// shared memory through descriptors in the canonical K-major layout without
-// swizzle (8-row x 16-byte core matrices).
+// A CTA walks output tiles of 128 voxels (one channel, 16 rows, 8 columns)
+// along the channel axis z, column of tiles after column of tiles.  Input
+// planes (the 18 x 10 halo of one channel) arrive one by one; plane i feeds
+// the three outputs z = i-1, i, i+1 with its taps kz = 2, 1, 0.  Their
+// accumulators D[128 voxels][32 features] lie side by side in tensor memory,
+// and the weights of the three kz side by side in shared memory, so one
+// tcgen05.mma (kind::f16, bfloat16 A and B, float32 D, M = 128, K = 16) with
+// N = 96 serves all three: 18 MMAs a tile (9 shifts in the plane x 2 steps of
+// K) where one per tap and output makes 54 of N = 32.  An MMA of N = 32 takes
+// as long as one of N = 96 (57 and 60 cycles measured): its time is the read
+// of the 4 KB A operand.  Every output still sums its 27 taps in the order kz,
+// ky, kx, K step.  The last layer, whose epilogue writes the prediction or the
+// loss terms, runs with 16 columns an output (N = 48).
 //
-// The tile's input halo (3 x 18 x 10 voxels) arrives by TMA: one
-// cp.async.bulk.tensor per 8-feature chunk, from a 4-D tensor map over
-// (8 features, x, y, z) of the [z][y][x][32] map (strides 64 B, 64 nx B,
-// 64 nx ny B; base offset 16 B per chunk).  A box lands as one chunk plane
-// [z][y][x][16 B], so the 8 consecutive voxels of an output row are one core
-// matrix in every tap's shifted window: rows of a window are 16 B apart, the
-// next output row (next 8-row group) is one halo row (160 B) further, the next
-// 8 input features one chunk plane further (planes padded to 8704 B, TMA wants
-// 128-byte aligned destinations).  Outside the cube the copy fills zeros: the
-// zero padding of the layer.  Weights are [tap][chunk][co][16 B] (next 8
-// outputs 128 B, next 8 inputs 512 B), loaded once per CTA.
+// Eight accumulators (256 of the 512 columns: two CTAs per SM) form a ring; an
+// MMA whose outputs run over its end is issued in two parts, and the first MMA
+// into a new accumulator is issued apart, without the accumulate flag.
 //
-// One halo buffer (90 KB of shared memory in all, two CTAs per SM): thread 0
-// issues tile i's MMAs (commit -> mbarrier mdone); once they have read the
-// halo, it issues the TMA of tile i+1 (mbarrier full), which then runs under
-// tile i's epilogue, while the SM's other CTA keeps the tensor core busy.
-// Every wait is bounded: on timeout the CTA records it in g_tc_timeouts,
-// waits (bounded) for its copy in flight, skips its remaining tiles and still
-// frees its tensor memory.
+// Roles: warps 4-7 load planes with 16-byte cp.async (zero fill outside the
+// cube: the zero padding of the layer) into a ring of shared-memory slots,
+// [chunk of 8 features][row][column][16 B] (the canonical K-major layout
+// without swizzle: 8 voxels of a row are one core matrix in every shifted
+// window; the chunk pitch of 2976 B spreads the chunks over the banks); warp
+// 8 issues the MMAs; warps 0-3 drain the accumulators.  (TMA boxes of 16-byte
+// rows, which this layout needs, move one 16-byte piece per two cycles and
+// fetch a 32-byte sector for each: they took 4300 of the 5150 cycles per tile
+// of a kernel that loaded each tile's halo so.)
+// Weights are [shift][chunk][2 - kz][co][16 B] (next 8 outputs 128 B, next 8
+// inputs 1536 B), loaded once per CTA.
+//
+// Every wait is bounded: a role that gives up records it in g_tc_timeouts and
+// leaves, the others run into their own bounds, and the CTA waits for its
+// copies and MMAs in flight (at the full bound) before it frees its tensor
+// memory.
 constexpr int U_TY = 16, U_TX = 8;                          // output tile: 16 rows x 8 columns, one channel
-constexpr int U_HY = U_TY + 2, U_HX = U_TX + 2;             // 18 x 10 halo per channel slice
-constexpr int U_HV = 3 * U_HY * U_HX;                       // 540 voxels
-constexpr int U_BOX = U_HV * 16;                            // bytes of one chunk box: 8640
-constexpr int U_CHUNK = 8704;                               // chunk plane stride (128-byte multiple)
-constexpr int U_HALO = 4 * U_CHUNK;                         // 34816
-constexpr int kLastN = 16;                                  // MMA width of the last layer (K <= 8 maps used)
+constexpr int U_HY = U_TY + 2, U_HX = U_TX + 2;             // 18 x 10 halo of a plane
+constexpr int Z_CH = 2976;                                  // chunk pitch of a plane slot (180 voxels x 16 B, padded)
+constexpr int Z_PLANE = 4 * Z_CH;                           // 11904
+constexpr int Z_NS = 4;                                     // plane slots
+constexpr int Z_PIECES = U_HY * U_HX * 4;                   // 16-byte pieces of a plane: 720
+constexpr int Z_RING = 8;                                   // accumulators
+constexpr int kLastN = 16;                                  // columns of an output of the last layer (K <= 8 maps used)
 template <int EPI> __host__ __device__ constexpr int epi_n() { return EPI >= EPI_PRED ? kLastN : C; }
-// weights: 55296 B (N = 32), 27648 B (N = 16); then 2 mbarriers and the TMEM address slot; alignment slack
+// weights: 55296 B (N = 32), 27648 B (N = 16); then the mbarriers and the TMEM address slot; alignment slack
 __host__ __device__ constexpr int u_w(int no) { return NTAP * 4 * no * 16; }
-__host__ __device__ constexpr int u_bar(int no) { return U_HALO + u_w(no); }
-__host__ __device__ constexpr int conv05_smem(int no) { return u_bar(no) + 64 + 128; }
+__host__ __device__ constexpr int u_bar(int no) { return Z_NS * Z_PLANE + u_w(no); }
+__host__ __device__ constexpr int conv05_smem(int no) { return u_bar(no) + 256 + 128; }
 // D f32, A/B bf16, both K-major, N = no, M = 128
 __host__ __device__ constexpr uint32_t idesc_bf16(int no) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(no >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
@@ -233,10 +241,6 @@ __device__ int g_tc_timeouts;
 // The drain waits after a give-up keep the full bound kWaitLimit, so that no
 // copy or MMA lands in shared or tensor memory after the CTA has left.
 __device__ long long g_wait_polls = kWaitLimit;
-
-struct HaloMaps {
-  CUtensorMap m[4];   // one per 8-feature chunk
-};
 
 __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
   uint64_t d = (uint64_t)((addr >> 4) & 0x3FFFu);
@@ -260,57 +264,82 @@ __device__ __forceinline__ bool mbar_wait_n(uint32_t bar, uint32_t parity, long 
   }
   return done != 0;
 }
-// pipeline wait: gives up after g_wait_polls polls
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  return mbar_wait_n(bar, parity, *(volatile long long*)&g_wait_polls);
+// Pipeline wait: gives up after `polls` polls, g_wait_polls as the kernel read
+// it once at its start (read at each wait, the load's latency, some 700 cycles,
+// stood in front of every poll).
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long polls) {
+  return mbar_wait_n(bar, parity, polls);
 }
 // drain wait after a give-up: the full bound
 __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) { return mbar_wait_n(bar, parity, kWaitLimit); }
 
-// Thread 0: the four chunk boxes of the tile at (x0, y0, z0) into halo buffer s_dst.
-__device__ __forceinline__ void issue_halo(const HaloMaps& maps, uint32_t s_dst, uint32_t bar, int x0, int y0,
-                                           int z0) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(4 * U_BOX) : "memory");
-#pragma unroll
-  for (int c = 0; c < 4; ++c)
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
-        "[%6];" ::"r"(s_dst + (uint32_t)(c * U_CHUNK)),
-        "l"(reinterpret_cast<uint64_t>(&maps.m[c])), "r"(0), "r"(x0 - 1), "r"(y0 - 1), "r"(z0 - 1), "r"(bar)
-        : "memory");
+__device__ __forceinline__ void tc_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// The run of output tiles of this CTA: tiles are numbered column by column
+// (z fastest) and split evenly.
+struct Runs {
+  long long at, end;
+  __device__ __forceinline__ Runs(int ncol, int nz) {
+    const long long total = (long long)ncol * nz;
+    at = total * blockIdx.x / gridDim.x;
+    end = total * (blockIdx.x + 1) / gridDim.x;
+  }
+  // next stretch za .. zb-1 of one column; false at the end
+  __device__ __forceinline__ bool next(int nz, int& col, int& za, int& zb) {
+    if (at >= end) return false;
+    col = (int)(at / nz);
+    za = (int)(at % nz);
+    const long long left = end - at;
+    zb = left < nz - za ? za + (int)left : nz;
+    at += zb - za;
+    return true;
+  }
+};
+
 template <int EPI>
-__global__ void __launch_bounds__(128)
-k_conv_tc05(const __grid_constant__ HaloMaps maps, const bf16* __restrict__ wk, const float* __restrict__ bias,
-            const bf16* __restrict__ mask, bf16* __restrict__ out, Dims d, int tiles_x, int tiles_y, int ntiles,
-            LastArgs la) {
+__global__ void __launch_bounds__(288, 2)
+k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const float* __restrict__ bias,
+            const bf16* __restrict__ mask, bf16* __restrict__ out, Dims d, int tiles_x, int tiles_y, LastArgs la) {
   constexpr int NO = epi_n<EPI>();
   constexpr bool kLast = EPI >= EPI_PRED;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ double s_red[32];
   const uint32_t s0 = (smem_u32(smem) + 127u) & ~127u;
-  const uint32_t s_halo = s0;
-  const uint32_t s_w = s0 + U_HALO;
-  const uint32_t s_full = s0 + u_bar(NO);         // TMA landed
-  const uint32_t s_done = s_full + 8;              // MMAs finished
-  const uint32_t s_tm = s_full + 16;               // TMEM address written by tcgen05.alloc
+  const uint32_t s_w = s0 + Z_NS * Z_PLANE;
+  const uint32_t s_full = s0 + u_bar(NO);          // plane loaded, per slot (128 loader threads)
+  const uint32_t s_free = s_full + 8 * Z_NS;       // plane's MMAs done, per slot
+  const uint32_t s_done = s_free + 8 * Z_NS;       // output complete, per accumulator
+  const uint32_t s_read = s_done + 8 * Z_RING;     // accumulator read (128 epilogue threads)
+  const uint32_t s_fin = s_read + 8 * Z_RING;      // everything the issuer started has finished
+  const uint32_t s_tm = s_fin + 8;                 // TMEM address written by tcgen05.alloc
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  // weights [tap][co][ci] -> [tap][chunk][co][16 B], once per CTA
+  // weights [tap][co][ci] -> [shift][chunk][2 - kz][co][16 B], once per CTA
   for (int i = threadIdx.x; i < NTAP * NO * 4; i += blockDim.x) {
-    const int c = i & 3, co = (i >> 2) % NO, t = i / (4 * NO);
-    cp_async16(s_w + (uint32_t)(((t * 4 + c) * NO + co) * 16), wk + (t * NO + co) * C + c * 8, 16);
+    const int c = i & 3, co = (i >> 2) % NO, t = i / (4 * NO), sh = t % 9, kz = t / 9;
+    cp_async16(s_w + (uint32_t)((((sh * 4 + c) * 3 + 2 - kz) * NO + co) * 16), wk + (t * NO + co) * C + c * 8, 16);
   }
   cp_async_wait_all();
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy writes, read by the MMA
   if (threadIdx.x == 0) {
-#pragma unroll
-    for (int b = 0; b < 2; ++b) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_full + 8 * b) : "memory");
+    for (int b = 0; b < Z_NS; ++b) {
+      muffin::mbar_init(s_full + 8 * b, 128);
+      muffin::mbar_init(s_free + 8 * b, 1);
+    }
+    for (int b = 0; b < Z_RING; ++b) {
+      muffin::mbar_init(s_done + 8 * b, 1);
+      muffin::mbar_init(s_read + 8 * b, 128);
+    }
+    muffin::mbar_init(s_fin, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 32;" ::"r"(s_tm) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(s_tm) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
@@ -319,173 +348,217 @@ k_conv_tc05(const __grid_constant__ HaloMaps maps, const bf16* __restrict__ wk, 
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(s_tm) : "memory");
 
-  float bn[NO];
-#pragma unroll
-  for (int c = 0; c < NO; ++c) bn[c] = (EPI != EPI_MASK && bias && (!kLast || c < la.K)) ? bias[c] : 0.f;
-  // last layer: input scale, and this thread's loss sums
-  const float sc = kLast ? *la.s : 1.f;
-  const float inv_sc = 1.0f / sc;
-  const double gs = 2.0 / (double)d.nvox;
-  const size_t plane = (size_t)d.ny * d.nx;
+  const long long polls = *(volatile long long*)&g_wait_polls;
+  Runs runs(tiles_x * tiles_y, d.nz);
+  int col, za, zb;
+  bool ok = true;
   double l2 = 0.0;
   double lsum[kMaxOut];
 #pragma unroll
   for (int k = 0; k < kMaxOut; ++k) lsum[k] = 0.0;
 
-  auto origin = [&](int tile, int& x0, int& y0, int& z0) {
-    const int txi = tile % tiles_x, rr = tile / tiles_x;
-    x0 = txi * U_TX;
-    y0 = (rr % tiles_y) * U_TY;
-    z0 = rr / tiles_y;
-  };
-  // thread 0 tracks the halo copy it may have in flight, so that an early
-  // exit can wait for it before the CTA's shared memory goes away
-  bool pending = false;
-  uint32_t pend_ph = 0;
-  // and the MMAs it committed but has not yet seen finish
-  bool mma_pending = false;
-  uint32_t mma_ph = 0;
-  if (threadIdx.x == 0 && (int)blockIdx.x < ntiles) {
-    int x0, y0, z0;
-    origin(blockIdx.x, x0, y0, z0);
-    issue_halo(maps, s_halo, s_full, x0, y0, z0);
-    pending = true;
-  }
-
-  int it = 0;
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
-    const uint32_t ph = (uint32_t)it & 1u;
-    int x0, y0, z0;
-    origin(tile, x0, y0, z0);
-    if (threadIdx.x == 0) {
-      if (mbar_wait(s_full, ph)) {
-        pending = false;
-        tc_fence_after();
-        const uint32_t hb = s_halo;
-        const uint32_t dt = tmem;
-#pragma unroll 1
-        for (int t = 0; t < NTAP; ++t) {
-          const int kz = t / 9, ky = (t / 3) % 3, kx = t % 3;
-          const uint32_t a0 = hb + (uint32_t)(((kz * U_HY + ky) * U_HX + kx) * 16);
-          const uint32_t b0 = s_w + (uint32_t)(t * 4 * NO * 16);
+  if (warp >= 4 && warp < 8) {
+    // ---------------- loaders: planes za-1 .. zb of each stretch, two planes in flight behind the newest
+    constexpr int NP = (Z_PIECES + 127) / 128;
+    const int tid = threadIdx.x - 128;
+    const unsigned char* base = reinterpret_cast<const unsigned char*>(in);
+    const size_t pitch = (size_t)d.ny * d.nx * ROWB;
+    int np = 0;                                     // planes issued so far
+    auto landed = [&](int p) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      mbar_arrive(s_full + 8 * (p % Z_NS));
+    };
+    while (ok && runs.next(d.nz, col, za, zb)) {
+      const int x0 = (col % tiles_x) * U_TX, y0 = (col / tiles_x) * U_TY;
+      uint32_t off[NP], dst[NP];
+      bool in_xy[NP];
 #pragma unroll
-          for (int kk = 0; kk < 2; ++kk) {
-            const uint64_t ad = umma_desc(a0 + kk * 2 * U_CHUNK, U_CHUNK, U_HX * 16);
-            const uint64_t bd = umma_desc(b0 + kk * 2 * NO * 16, NO * 16, 8 * 16);
-            const uint32_t acc = (t | kk) != 0;
-            asm volatile(
-                "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(dt),
-                "l"(ad), "l"(bd), "r"(idesc_bf16(NO)), "r"(acc)
-                : "memory");
-          }
+      for (int i = 0; i < NP; ++i) {
+        const int id = tid + 128 * i, c = id & 3, v = id >> 2, hx = v % U_HX, hy = v / U_HX;
+        const int gy = y0 - 1 + hy, gx = x0 - 1 + hx;
+        in_xy[i] = (unsigned)gy < (unsigned)d.ny && (unsigned)gx < (unsigned)d.nx;
+        off[i] = in_xy[i] ? ((uint32_t)gy * (uint32_t)d.nx + (uint32_t)gx) * ROWB + c * 16 : 0u;
+        dst[i] = (uint32_t)(c * Z_CH + v * 16);
+      }
+      for (int z = za - 1; z <= zb; ++z) {
+        const int slot = np % Z_NS;
+        if (!mbar_wait(s_free + 8 * slot, (uint32_t)(np / Z_NS & 1) ^ 1u, polls)) { ok = false; break; }
+        const bool in_z = (unsigned)z < (unsigned)d.nz;
+        const unsigned char* pl = base + (in_z ? (size_t)z * pitch : 0);
+        const uint32_t sp = s0 + slot * Z_PLANE;
+#pragma unroll
+        for (int i = 0; i < NP; ++i)
+          if (tid + 128 * i < Z_PIECES) cp_async16(sp + dst[i], pl + off[i], in_z && in_xy[i] ? 16 : 0);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (np >= 2) {
+          asm volatile("cp.async.wait_group 2;" ::: "memory");
+          landed(np - 2);
         }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s_done)
-                     : "memory");
-        mma_pending = true;
-        mma_ph = ph;
+        ++np;
       }
     }
-    const bool done = mbar_wait(s_done, ph);
-    if (threadIdx.x == 0 && done) mma_pending = false;
-    if (__syncthreads_or(!done)) {          // one decision for the whole block
-      if (threadIdx.x == 0) atomicAdd(&g_tc_timeouts, 1);
-      break;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (ok) {
+      if (np >= 2) landed(np - 2);
+      if (np >= 1) landed(np - 1);
     }
-    // the MMAs have read the halo: the next tile's copy runs under this epilogue
-    if (threadIdx.x == 0 && tile + (int)gridDim.x < ntiles) {
-      int nx0, ny0, nz0;
-      origin(tile + gridDim.x, nx0, ny0, nz0);
-      issue_halo(maps, s_halo, s_full, nx0, ny0, nz0);
-      pending = true;
-      pend_ph = (uint32_t)(it + 1) & 1u;
-    }
-    tc_fence_after();
-    // row m = 32 warp + lane of D is output voxel (y0 + m / 8, x0 + m % 8) of channel z0
-    const int m = warp * 32 + lane;
-    const int z = z0, y = y0 + (m >> 3), x = x0 + (m & 7);
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-    if constexpr (!kLast) {
-      uint32_t r[C];
+  } else if (warp == 8) {
+    // ---------------- issuer
+    int np = 0, no = 0;                             // planes taken, outputs finished before this stretch
+    const uint64_t wd0 = umma_desc(s_w, 3 * NO * 16, 8 * 16);
+    // MMA of shift / K step (its offsets within the plane and the weights) into nb accumulators from ring block
+    // blk on, weight blocks from b0 on
+    auto mma = [&](uint64_t ad, uint64_t wd, int blk, int nb, int b0, uint32_t accum) {
       asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-          "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-            "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-            "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-          : "r"(taddr));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (inside(d, z, y, x)) {
-        const size_t base = vox(d, z, y, x) * C;
-        float v[C];
+          "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+          "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (uint32_t)(blk * NO)),
+          "l"(ad), "l"(wd + (uint64_t)(b0 * NO)), "r"(idesc_bf16(nb * NO)), "r"(accum)
+          : "memory");
+    };
+    while (lane == 0 && ok && runs.next(d.nz, col, za, zb)) {
+      const int n = zb - za;
+      for (int i = 0; i < n + 2; ++i) {             // plane za - 1 + i feeds outputs i-2 .. i of the stretch
+        const int slot = np % Z_NS;
+        const int lo = i < 2 ? 0 : i - 2, hi = i < n ? i : n - 1;
+        if (!mbar_wait(s_full + 8 * slot, (uint32_t)(np / Z_NS & 1), polls)) { ok = false; break; }
+        if (i < n) {                                // output i starts here: its accumulator must have been read
+          const int o = no + i;
+          if (!mbar_wait(s_read + 8 * (o % Z_RING), (uint32_t)(o / Z_RING & 1) ^ 1u, polls)) { ok = false; break; }
+        }
+        tc_fence_after();
+        // outputs lo .. hi as one or two runs of the ring
+        const int blk = (no + lo) % Z_RING, nb = hi - lo + 1, b0 = lo - (i - 2);
+        const int n1 = blk + nb > Z_RING ? Z_RING - blk : nb;
+        const uint64_t ad0 = umma_desc(s0 + slot * Z_PLANE, Z_CH, U_HX * 16);
+        // first shift and step: a new output's accumulator is overwritten
+        if (i < n) {
+          if (nb > 1) {
+            const int m1 = n1 < nb ? n1 : nb - 1;
+            mma(ad0, wd0, blk, m1, b0, 1u);
+            if (nb - 1 > m1) mma(ad0, wd0, 0, nb - 1 - m1, b0 + m1, 1u);
+          }
+          mma(ad0, wd0, (no + i) % Z_RING, 1, 2, 0u);
+        } else {
+          mma(ad0, wd0, blk, n1, b0, 1u);
+          if (n1 < nb) mma(ad0, wd0, 0, nb - n1, b0 + n1, 1u);
+        }
 #pragma unroll
-        for (int c = 0; c < C; ++c) v[c] = __uint_as_float(r[c]);
-        if (EPI == EPI_MASK) {
-          if (mask) {
-            const uint4* mp = reinterpret_cast<const uint4*>(mask + base);
+        for (int q = 1; q < 18; ++q) {
+          const int sh = q >> 1, kk = q & 1;
+          const uint64_t ad = ad0 + (uint64_t)((sh / 3) * U_HX + sh % 3 + kk * 2 * (Z_CH / 16));
+          const uint64_t wd = wd0 + (uint64_t)((sh * 4 + kk * 2) * 3 * NO);
+          mma(ad, wd, blk, n1, b0, 1u);
+          if (n1 < nb) mma(ad, wd, 0, nb - n1, b0 + n1, 1u);
+        }
+        tc_commit(s_free + 8 * slot);
+        ++np;
+        if (i >= 2) tc_commit(s_done + 8 * ((no + i - 2) % Z_RING));
+      }
+      no += n;
+    }
+    if (lane == 0) tc_commit(s_fin);
+    __syncwarp();
+  } else if (warp < 4) {
+    // ---------------- epilogue: row m = 32 warp + lane of D is voxel (y0 + m / 8, x0 + m % 8)
+    float bn[NO];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              float mf[8];
-              unpack8(mp[q], mf);
-#pragma unroll
-              for (int e = 0; e < 8; ++e)
-                if (!(mf[e] > 0.f)) v[8 * q + e] = 0.f;
+    for (int c = 0; c < NO; ++c) bn[c] = (EPI != EPI_MASK && bias && (!kLast || c < la.K)) ? bias[c] : 0.f;
+    // last layer: input scale
+    const float sc = kLast ? *la.s : 1.f;
+    const float inv_sc = 1.0f / sc;
+    const double gs = 2.0 / (double)d.nvox;
+    const size_t plane = (size_t)d.ny * d.nx;
+    const int m = warp * 32 + lane;
+    int no = 0;
+    while (ok && runs.next(d.nz, col, za, zb)) {
+      const int x = (col % tiles_x) * U_TX + (m & 7), y = (col / tiles_x) * U_TY + (m >> 3);
+      for (int z = za; z < zb; ++z, ++no) {
+        const int acc = no % Z_RING;
+        if (!mbar_wait(s_done + 8 * acc, (uint32_t)(no / Z_RING & 1), polls)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t taddr = tmem + (uint32_t)(acc * NO) + ((uint32_t)(warp * 32) << 16);
+        if constexpr (!kLast) {
+          uint32_t r[C];
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+              "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+              : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+                "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+              : "r"(taddr));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          tc_fence_before();
+          mbar_arrive(s_read + 8 * acc);
+          if (inside(d, z, y, x)) {
+            const size_t base = vox(d, z, y, x) * C;
+            float v[C];
+    #pragma unroll
+            for (int c = 0; c < C; ++c) v[c] = __uint_as_float(r[c]);
+            if (EPI == EPI_MASK) {
+              if (mask) {
+                const uint4* mp = reinterpret_cast<const uint4*>(mask + base);
+    #pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                  float mf[8];
+                  unpack8(mp[q], mf);
+    #pragma unroll
+                  for (int e = 0; e < 8; ++e)
+                    if (!(mf[e] > 0.f)) v[8 * q + e] = 0.f;
+                }
+              }
+            } else {
+    #pragma unroll
+              for (int c = 0; c < C; ++c) {
+                v[c] += bn[c];
+                if (EPI == EPI_RELU) v[c] = fmaxf(v[c], 0.f);
+              }
             }
+            uint4* o = reinterpret_cast<uint4*>(out + base);
+    #pragma unroll
+            for (int q = 0; q < 4; ++q) o[q] = pack8(v + 8 * q);
           }
         } else {
-#pragma unroll
-          for (int c = 0; c < C; ++c) {
-            v[c] += bn[c];
-            if (EPI == EPI_RELU) v[c] = fmaxf(v[c], 0.f);
-          }
-        }
-        uint4* o = reinterpret_cast<uint4*>(out + base);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) o[q] = pack8(v + 8 * q);
-      }
-    } else {
-      // last layer: z_k = D[m][k] + b_k for the K maps (columns K .. 15 hold zero weights)
-      uint32_t r[kLastN];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-          : "r"(taddr));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (inside(d, z, y, x)) {
-        const int K = la.K;
-        const size_t v = vox(d, z, y, x);
-        const size_t a0 = ((size_t)z * (K > 1 ? K - 1 : 1)) * plane + (size_t)y * d.nx + x;
-#pragma unroll
-        for (int k = 0; k < kMaxOut; ++k) {
-          if (k < K) {
-            const float zk = __uint_as_float(r[k]) + bn[k];
-            if constexpr (EPI == EPI_LOSS) {
-              const float tk = k == 0 ? la.tx[v] * inv_sc : __bfloat162float(la.taux[a0 + (size_t)(k - 1) * plane]);
-              const float rk = zk - tk;
-              la.d6[v * K + k] = (float)(gs * la.lam.v[k]) * rk;
-              l2 += (double)la.lam.v[k] * rk * rk;
-              lsum[k] += rk;
-            } else {
-              if (k == 0) la.out_x[v] = fmaxf(sc * zk, 0.f);
-              else la.out_aux[a0 + (size_t)(k - 1) * plane] = fminf(fmaxf(zk, -1.f), 1.f);
+          // last layer: z_k = D[m][k] + b_k for the K maps (columns K .. 15 hold zero weights)
+          uint32_t r[kLastN];
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+              : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+              : "r"(taddr));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          tc_fence_before();
+          mbar_arrive(s_read + 8 * acc);
+          if (inside(d, z, y, x)) {
+            const int K = la.K;
+            const size_t v = vox(d, z, y, x);
+            const size_t a0 = ((size_t)z * (K > 1 ? K - 1 : 1)) * plane + (size_t)y * d.nx + x;
+    #pragma unroll
+            for (int k = 0; k < kMaxOut; ++k) {
+              if (k < K) {
+                const float zk = __uint_as_float(r[k]) + bn[k];
+                if constexpr (EPI == EPI_LOSS) {
+                  const float tk = k == 0 ? la.tx[v] * inv_sc : __bfloat162float(la.taux[a0 + (size_t)(k - 1) * plane]);
+                  const float rk = zk - tk;
+                  la.d6[v * K + k] = (float)(gs * la.lam.v[k]) * rk;
+                  l2 += (double)la.lam.v[k] * rk * rk;
+                  lsum[k] += rk;
+                } else {
+                  if (k == 0) la.out_x[v] = fmaxf(sc * zk, 0.f);
+                  else la.out_aux[a0 + (size_t)(k - 1) * plane] = fminf(fmaxf(zk, -1.f), 1.f);
+                }
+              }
             }
           }
         }
       }
     }
-    tc_fence_before();
-    __syncthreads();     // the accumulator is read before the next tile's MMAs overwrite it
-    tc_fence_after();
   }
-  // only after a give-up: the copy and the MMAs still in flight land before the CTA leaves
-  if (threadIdx.x == 0 && pending) mbar_drain(s_full, pend_ph);
-  if (threadIdx.x == 0 && mma_pending) mbar_drain(s_done, mma_ph);
+  const bool fin = mbar_drain(s_fin, 0);   // every copy and MMA issued, also after a give-up: TMEM is freed below
   tc_fence_before();
-  __syncthreads();
+  if (__syncthreads_or(!ok || !fin) && threadIdx.x == 0) atomicAdd(&g_tc_timeouts, 1);
   tc_fence_after();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 32;" ::"r"(tmem) : "memory");
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
   if constexpr (EPI == EPI_LOSS) {
     // lpart[block] = (sum_k lam_k sum_p r_k^2, sum_p r_0, ..., sum_p r_{K-1}), fixed order
     const double t2 = muffin::block_sum(l2, s_red);
@@ -594,6 +667,7 @@ k_wgrad_tc05(const __grid_constant__ WgradMaps maps, float* __restrict__ part, f
     y0 = (rr % tiles_y) * U_TY;
     z0 = rr / tiles_y;
   };
+  const long long polls = *(volatile long long*)&g_wait_polls;
   const int nmine = ntiles > (int)blockIdx.x ? (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
   bool ok = true;
   float bacc = 0.f;
@@ -611,7 +685,7 @@ k_wgrad_tc05(const __grid_constant__ WgradMaps maps, float* __restrict__ part, f
     for (int it = 0; it < nmine && ok; ++it) {
       const int s = it % WG_NS;
       const uint32_t ph = (uint32_t)(it / WG_NS) & 1u;
-      if (!mbar_wait(s_full + 8 * s, ph)) { ok = false; break; }
+      if (!mbar_wait(s_full + 8 * s, ph, polls)) { ok = false; break; }
       tc_fence_after();
       const uint32_t sa = s0 + s * WG_STAGE, sb = sa + WG_A;
 #pragma unroll 1
@@ -635,7 +709,7 @@ k_wgrad_tc05(const __grid_constant__ WgradMaps maps, float* __restrict__ part, f
       if (it >= 1 && it - 1 + WG_NS < nmine) {
         const int sp = (it - 1) % WG_NS;
         const uint32_t pp = (uint32_t)((it - 1) / WG_NS) & 1u;
-        if (!mbar_wait(s_done + 8 * sp, pp) || !mbar_wait(s_freed + 8 * sp, pp)) { ok = false; break; }
+        if (!mbar_wait(s_done + 8 * sp, pp, polls) || !mbar_wait(s_freed + 8 * sp, pp, polls)) { ok = false; break; }
         int x0, y0, z0;
         origin(blockIdx.x + (it - 1 + WG_NS) * gridDim.x, x0, y0, z0);
         wg_issue(maps, s0 + sp * WG_STAGE, s_full + 8 * sp, x0, y0, z0);
@@ -652,7 +726,7 @@ k_wgrad_tc05(const __grid_constant__ WgradMaps maps, float* __restrict__ part, f
     for (int it = 0; it < nmine && ok; ++it) {
       const int s = it % WG_NS;
       const uint32_t ph = (uint32_t)(it / WG_NS) & 1u;
-      if (!mbar_wait(s_full + 8 * s, ph)) { ok = false; break; }
+      if (!mbar_wait(s_full + 8 * s, ph, polls)) { ok = false; break; }
       const unsigned char* b = smem + (s0 - smem_u32(smem)) + s * WG_STAGE + WG_A;
       const int c = lane >> 3, e = lane & 7;
 #pragma unroll 8
@@ -1172,23 +1246,6 @@ EncodeTiledFn encode_tiled() {
   return fn;
 }
 
-// The four 4-D tensor maps (8 features, x, y, z) of a [z][y][x][32] bfloat16 map, one per chunk.
-cudaError_t halo_maps(const bf16* in, const Dims& d, HaloMaps* maps) {
-  EncodeTiledFn enc = encode_tiled();
-  if (!enc) return cudaErrorNotSupported;
-  const cuuint64_t dims[4] = {8, (cuuint64_t)d.nx, (cuuint64_t)d.ny, (cuuint64_t)d.nz};
-  const cuuint64_t strides[3] = {(cuuint64_t)C * 2, (cuuint64_t)d.nx * C * 2, (cuuint64_t)d.ny * d.nx * C * 2};
-  const cuuint32_t box[4] = {8, U_HX, U_HY, 3};
-  const cuuint32_t estr[4] = {1, 1, 1, 1};
-  for (int c = 0; c < 4; ++c) {
-    const CUresult r = enc(&maps->m[c], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)(in + c * 8), dims, strides,
-                           box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                           CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-  }
-  return cudaSuccess;
-}
-
 // A host-side failure of a layer launch (a tensor map that could not be
 // encoded), reported by the next status check of the calling entry point.
 cudaError_t g_launch_err = cudaSuccess;
@@ -1215,16 +1272,9 @@ int tc05_grid(const Dims& d, int sms) {
 template <int EPI>
 cudaError_t launch_tc05(const bf16* in, const bf16* wk, const float* bias, const bf16* mask, bf16* out,
                         const Dims& d, int sms, cudaStream_t st, const LastArgs& la) {
-  HaloMaps maps;
-  const cudaError_t e = halo_maps(in, d, &maps);
-  if (e != cudaSuccess) {
-    g_launch_err = e;
-    return e;
-  }
   int tx, ty;
-  const int ntiles = tc05_tiles(d, tx, ty);
-  k_conv_tc05<EPI><<<tc05_grid(d, sms), 128, conv05_smem(epi_n<EPI>()), st>>>(maps, wk, bias, mask, out, d, tx, ty,
-                                                                             ntiles, la);
+  tc05_tiles(d, tx, ty);
+  k_conv_tc05<EPI><<<tc05_grid(d, sms), 288, conv05_smem(epi_n<EPI>()), st>>>(in, wk, bias, mask, out, d, tx, ty, la);
   return cudaGetLastError();
 }
 
