@@ -5,8 +5,8 @@
 // fields of its state (the planes of the wavelet dual U).
 //
 // Feature maps are [nz][ny][nx][32] bfloat16 (64 bytes per voxel).  The
-// tensor-core kernels (below) walk tiles of 1 x 16 x 8 voxels whose halos
-// arrive by TMA.  The CUDA-core kernels work on output tiles of 2 x 8 x 16
+// tensor-core kernels (below) march tiles of 1 x 16 x 8 voxels along the
+// channel axis.  The CUDA-core kernels work on output tiles of 2 x 8 x 16
 // voxels (channel, row, column) whose inputs, with a one-voxel halo
 // (4 x 10 x 18), are staged in shared memory by cp.async with zero fill
 // outside the cube (the zero padding of the layers); there a voxel's 64 bytes
@@ -22,15 +22,14 @@
 //   input grad   da[p][ci] = sum_tap sum_co dz[p - d(tap)][co] W[tap][co][ci],
 //                 the same kernel on the flipped, transposed weights,
 //   weight grad  dW[tap][co][ci] = sum_p dz[p][co] a[p + d(tap)][ci]
-//                 (M = (row offset, ci), N = co, K = voxels), tcgen05.mma with nine
-//                 accumulators resident in tensor memory for the CTA's whole run.
+//                 (M = (row offset, ci), N = (channel offset, co), K = voxels), tcgen05.mma
+//                 with the accumulators resident in tensor memory for the CTA's whole run.
 // The last layer's forward (prediction, or the loss and its gradient d6) is
 // the same tcgen05 kernel with N = 16 (weights of maps K .. 15 zero).  The
 // 1 -> 32 layer and the last layer's gradients (27 or 864 multiply-adds per
 // voxel and output, with float32 d6) run on the CUDA cores.  Every reduction
 // over voxels is a per-block partial sum followed by a fixed-order sum:
 // results do not depend on scheduling.
-#include <cuda.h>            // CUtensorMap (the encoder is reached through the runtime's driver entry point)
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -573,82 +572,69 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
   }
 }
 
-// ------------------------------------------------------------------ 32 -> 32 weight gradient on tcgen05, fed by TMA
+// ------------------------------------------------------------------ 32 -> 32 weight gradient on tcgen05, marching along z
 //
 // dW[tap][co][ci] = sum_p dz[p][co] a[p + d(tap)][ci] as tensor-core products
-// D[m][n] += A[m][k] B[k][n] with k = output voxel p, n = co and
-// m = (ky, ci): one 128-row accumulator per (kz, kx) holds the three row
-// offsets ky = 0..2 of the tap (rows 96..127, "ky = 3", are computed and
-// dropped).  Nine accumulators of 32 float32 columns stay in tensor memory for
-// the CTA's whole run over its tiles; the sums leave TMEM once, at the end.
+// D[m][n] += A[m][k] B[k][n] with k = voxel of a tile of one channel,
+// m = (ky, ci) and n = (2 - kz, co): the plane zi of a is multiplied with the
+// dz planes zi - 1, zi, zi + 1 at once (kz = 2, 1, 0), so one accumulator of
+// 128 x 96 per kx holds the nine row and channel offsets of its taps (rows
+// 96..127, "ky = 3", are computed and dropped).  The three accumulators (288
+// columns) stay in tensor memory for the CTA's whole run over its tiles; the
+// sums leave TMEM once, at the end.  24 MMAs of N = 96 per tile replace 72 of
+// N = 32; an MMA takes as long either way (the read of its A operand).
 //
 // Both operands are MN-major (M or N contiguous: the 8 features of a chunk),
-// canonical layout without swizzle: core matrices of 8 voxels x 16 bytes.
-// The input halo of a tile (3 x 19 x 10 voxels: rows y0-1 .. y0+17, the last
-// one only feeding the dropped rows) lands by one TMA copy as
-// [y][chunk][z][x][16 B] (a 5-D tensor map over (8 features, x, z, chunk, y)
-// with a 16-byte chunk stride): the next 8 rows of m (next chunk, or next ky
-// after four chunks) are 480 B apart, the next 8 voxels of k (next output
-// row) 1920 B.  The tile's own dz lands as [y][chunk][x][16 B]: next 8 co
-// 128 B, next 8 voxels 512 B.
+// canonical layout without swizzle: core matrices of 8 voxels x 16 bytes.  A
+// plane of a with its halo (rows y0-1 .. y0+17, the last one only feeding the
+// dropped rows) is [row][chunk][column][16 B]: the next 8 rows of m (next
+// chunk, or next ky after four) are 160 B apart, the next 8 voxels of k (next
+// row) 640 B.  The dz tiles of eight channels form a ring
+// [row][ring slot][chunk][column][16 B], so that consecutive channels continue
+// n: next 8 of n 128 B, next 8 voxels 4096 B; MMAs that run over the ring's end
+// are issued in two parts.
 //
-// Thread 0 keeps a three-stage TMA ring ahead of its MMAs (72 per tile:
-// 9 accumulators x 8 steps of K = 16); warp 1 sums the dz tiles into the bias
-// gradient as they land and releases each stage through an mbarrier.  One CTA
-// per SM (the ring takes 146 KB of shared memory; the accumulators take all
-// 512 TMEM columns).  Every wait is bounded; a CTA that gives up records it in
-// g_tc_timeouts, waits (bounded) for its copies and MMAs in flight, writes
-// nothing and frees its tensor memory.
-constexpr int WG_HY = U_TY + 3;                        // 19 halo rows (one extra for the dropped rows)
-constexpr int WG_A = WG_HY * 4 * 3 * U_HX * 16;        // 36480 B: [19][4][3][10][16 B]
-constexpr int WG_ROW = 4 * 3 * U_HX * 16;              // 1920 B per halo row
-constexpr int WG_B = U_TY * 4 * U_TX * 16;             // 8192 B: [16][4][8][16 B]
-constexpr int WG_STAGE = WG_A + WG_B;                  // 44672 B (a multiple of 128)
-constexpr int WG_NS = 3;                               // ring stages
-constexpr int WG_SLACK = 16384;                        // room past the ring that no descriptor layout can leave
-constexpr int WG_BAR = WG_NS * WG_STAGE + WG_SLACK;    // full[3], done[3], freed[3], fin, TMEM slot
-constexpr int wgrad05_smem = WG_BAR + 128 + 128;
-// D f32, A/B bf16, both MN-major, N = 32, M = 128
-constexpr uint32_t kIdescWgrad = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                                 ((uint32_t)(C >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
-
-struct WgradMaps {
-  CUtensorMap a;    // (8, x, z, chunk, y) of the layer input
-  CUtensorMap dz;   // (8, x, chunk, y, z) of the output gradient
-};
-
-__device__ __forceinline__ void wg_issue(const WgradMaps& maps, uint32_t stage, uint32_t bar, int x0, int y0, int z0) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(WG_STAGE) : "memory");
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
-      "[%7];" ::"r"(stage),
-      "l"(reinterpret_cast<uint64_t>(&maps.a)), "r"(0), "r"(x0 - 1), "r"(z0 - 1), "r"(0), "r"(y0 - 1), "r"(bar)
-      : "memory");
-  asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
-      "[%7];" ::"r"(stage + WG_A),
-      "l"(reinterpret_cast<uint64_t>(&maps.dz)), "r"(0), "r"(x0), "r"(0), "r"(y0), "r"(z0), "r"(bar)
-      : "memory");
+// Roles: warps 4-7 load with 16-byte cp.async (zero fill outside the cube),
+// warp 8 issues the MMAs, warps 0-3 sum the dz tiles into the bias gradient
+// as they land and store the sums at the end.  One CTA per SM.  Every wait is
+// bounded; a CTA that gives up records it in g_tc_timeouts, waits (bounded) for
+// its copies and MMAs in flight, writes nothing and frees its tensor memory.
+constexpr int WG_HY = U_TY + 3;                        // 19 rows (one extra for the dropped ones)
+constexpr int WG_CH = U_HX * 16;                       // chunk pitch 160 B
+constexpr int WG_ROW = 4 * WG_CH;                      // row pitch 640 B
+constexpr int WG_A = WG_HY * WG_ROW;                   // 12160 B
+constexpr int WG_NS = 4;                               // slots of a planes
+constexpr int WG_R = 8;                                // ring of dz tiles (more than WG_NS + 2)
+constexpr int WG_DROW = WG_R * 4 * U_TX * 16;          // row pitch of the ring 4096 B
+constexpr int WG_B = U_TY * WG_DROW;                   // 65536 B
+constexpr int WG_BAR = WG_NS * WG_A + WG_B;            // full, free, fin, TMEM slot
+constexpr int wgrad05_smem = 120 * 1024;               // more than half an SM: one CTA holds all of the tensor memory
+static_assert(WG_BAR + 256 + 128 <= wgrad05_smem, "weight gradient shared memory");
+constexpr int WG_N = 3 * C;
+// D f32, A/B bf16, both MN-major, N = n, M = 128
+__host__ __device__ constexpr uint32_t idesc_wgrad(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) |
+         ((uint32_t)(128 >> 4) << 24);
 }
 
-__global__ void __launch_bounds__(128)
-k_wgrad_tc05(const __grid_constant__ WgradMaps maps, float* __restrict__ part, float* __restrict__ bpart, Dims d,
-             int tiles_x, int tiles_y, int ntiles) {
+__global__ void __launch_bounds__(288, 1)
+k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __restrict__ part,
+             float* __restrict__ bpart, Dims d, int tiles_x, int tiles_y) {
   extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ float s_b[128 * 8];
   const uint32_t s0 = (smem_u32(smem) + 127u) & ~127u;
-  const uint32_t s_full = s0 + WG_BAR;          // TMA landed, per stage
-  const uint32_t s_done = s_full + 8 * WG_NS;   // MMAs of the stage's tile finished
-  const uint32_t s_freed = s_done + 8 * WG_NS;  // warp 1 has read the stage's dz
-  const uint32_t s_fin = s_freed + 8 * WG_NS;   // every MMA of the CTA finished
+  const uint32_t s_dz = s0 + WG_NS * WG_A;
+  const uint32_t s_full = s0 + WG_BAR;          // plane and dz tile loaded, per slot (128 loader threads)
+  const uint32_t s_free = s_full + 8 * WG_NS;   // MMAs done and dz summed, per slot (1 + 128 threads)
+  const uint32_t s_fin = s_free + 8 * WG_NS;    // every MMA of the CTA finished
   const uint32_t s_tm = s_fin + 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int b = 0; b < WG_NS; ++b) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_full + 8 * b) : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_done + 8 * b) : "memory");
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 32;" ::"r"(s_freed + 8 * b) : "memory");
+      muffin::mbar_init(s_full + 8 * b, 128);
+      muffin::mbar_init(s_free + 8 * b, 129);
     }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(s_fin) : "memory");
+    muffin::mbar_init(s_fin, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -660,80 +646,151 @@ k_wgrad_tc05(const __grid_constant__ WgradMaps maps, float* __restrict__ part, f
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(s_tm) : "memory");
+  if (warp < 4) {                               // accumulators start at zero
+    const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16);
+    for (int c = 0; c < 3 * WG_N; c += 8)
+      asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(ta + (uint32_t)c),
+                   "r"(0u)
+                   : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
 
-  auto origin = [&](int tile, int& x0, int& y0, int& z0) {
-    const int txi = tile % tiles_x, rr = tile / tiles_x;
-    x0 = txi * U_TX;
-    y0 = (rr % tiles_y) * U_TY;
-    z0 = rr / tiles_y;
-  };
   const long long polls = *(volatile long long*)&g_wait_polls;
-  const int nmine = ntiles > (int)blockIdx.x ? (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+  Runs runs(tiles_x * tiles_y, d.nz);
+  int col, za, zb;
   bool ok = true;
-  float bacc = 0.f;
-  if (threadIdx.x == 0) {
-    // per stage: bit b of `used` once a copy was issued into it, bit b of
-    // `odd` the parity of the number of copies (what an early exit waits for)
-    uint32_t used = 0, odd = 0;
-    for (int i = 0; i < WG_NS && i < nmine; ++i) {
-      int x0, y0, z0;
-      origin(blockIdx.x + i * gridDim.x, x0, y0, z0);
-      wg_issue(maps, s0 + i * WG_STAGE, s_full + 8 * i, x0, y0, z0);
-      used |= 1u << i;
-      odd ^= 1u << i;
-    }
-    for (int it = 0; it < nmine && ok; ++it) {
-      const int s = it % WG_NS;
-      const uint32_t ph = (uint32_t)(it / WG_NS) & 1u;
-      if (!mbar_wait(s_full + 8 * s, ph, polls)) { ok = false; break; }
-      tc_fence_after();
-      const uint32_t sa = s0 + s * WG_STAGE, sb = sa + WG_A;
-#pragma unroll 1
-      for (int acc = 0; acc < 9; ++acc) {
-        const int kz = acc / 3, kx = acc % 3;
+  float bacc[8];
 #pragma unroll
-        for (int rp = 0; rp < U_TY / 2; ++rp) {
-          const uint64_t ad = umma_desc(sa + (uint32_t)(2 * rp * WG_ROW + kz * U_HX * 16 + kx * 16), WG_ROW, 3 * U_HX * 16);
-          const uint64_t bd = umma_desc(sb + (uint32_t)(2 * rp * 4 * U_TX * 16), 4 * U_TX * 16, U_TX * 16);
-          const uint32_t accum = (it | rp) != 0;
+  for (int e = 0; e < 8; ++e) bacc[e] = 0.f;
+
+  if (warp >= 4 && warp < 8) {
+    // ---------------- loaders: step i of a stretch brings plane za - 1 + i of a and dz tile za + i
+    constexpr int NA = (WG_HY * U_HX * 4 + 127) / 128, ND = U_TY * U_TX * 4 / 128;
+    const int tid = threadIdx.x - 128;
+    const unsigned char *pa = reinterpret_cast<const unsigned char*>(a), *pd = reinterpret_cast<const unsigned char*>(dz);
+    const size_t pitch = (size_t)d.ny * d.nx * ROWB;
+    int np = 0, no = 0;
+    auto landed = [&](int p) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      mbar_arrive(s_full + 8 * (p % WG_NS));
+    };
+    while (ok && runs.next(d.nz, col, za, zb)) {
+      const int x0 = (col % tiles_x) * U_TX, y0 = (col / tiles_x) * U_TY, n = zb - za;
+      uint32_t aoff[NA], adst[NA], doff[ND], ddst[ND];
+      bool ain[NA], din[ND];
+#pragma unroll
+      for (int i = 0; i < NA; ++i) {
+        const int id = tid + 128 * i, c = id & 3, v = id >> 2, hx = v % U_HX, hy = v / U_HX;
+        const int gy = y0 - 1 + hy, gx = x0 - 1 + hx;
+        ain[i] = (unsigned)gy < (unsigned)d.ny && (unsigned)gx < (unsigned)d.nx;
+        aoff[i] = ain[i] ? ((uint32_t)gy * (uint32_t)d.nx + (uint32_t)gx) * ROWB + c * 16 : 0u;
+        adst[i] = (uint32_t)(hy * WG_ROW + c * WG_CH + hx * 16);
+      }
+#pragma unroll
+      for (int i = 0; i < ND; ++i) {
+        const int id = tid + 128 * i, x = id & 7, c = (id >> 3) & 3, y = id >> 5;
+        const int gy = y0 + y, gx = x0 + x;
+        din[i] = gy < d.ny && gx < d.nx;
+        doff[i] = din[i] ? ((uint32_t)gy * (uint32_t)d.nx + (uint32_t)gx) * ROWB + c * 16 : 0u;
+        ddst[i] = (uint32_t)(y * WG_DROW + (c * U_TX + x) * 16);
+      }
+      for (int i = 0; i < n + 2; ++i) {
+        const int slot = np % WG_NS, z = za - 1 + i;
+        if (!mbar_wait(s_free + 8 * slot, (uint32_t)(np / WG_NS & 1) ^ 1u, polls)) { ok = false; break; }
+        const bool in_z = (unsigned)z < (unsigned)d.nz;
+        const unsigned char* pl = pa + (in_z ? (size_t)z * pitch : 0);
+        const uint32_t sp = s0 + slot * WG_A;
+#pragma unroll
+        for (int q = 0; q < NA; ++q)
+          if (tid + 128 * q < WG_HY * U_HX * 4) cp_async16(sp + adst[q], pl + aoff[q], in_z && ain[q] ? 16 : 0);
+        if (i < n) {
+          const unsigned char* pz = pd + (size_t)(za + i) * pitch;
+          const uint32_t sd = s_dz + (uint32_t)((no + i) % WG_R) * (4 * U_TX * 16);
+#pragma unroll
+          for (int q = 0; q < ND; ++q) cp_async16(sd + ddst[q], pz + doff[q], din[q] ? 16 : 0);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (np >= 2) {
+          asm volatile("cp.async.wait_group 2;" ::: "memory");
+          landed(np - 2);
+        }
+        ++np;
+      }
+      no += n;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    if (ok) {
+      if (np >= 2) landed(np - 2);
+      if (np >= 1) landed(np - 1);
+    }
+  } else if (warp == 8) {
+    // ---------------- issuer: plane i of a stretch with the dz tiles lo .. hi = i-2 .. i
+    int np = 0, no = 0;
+    while (lane == 0 && ok && runs.next(d.nz, col, za, zb)) {
+      const int n = zb - za;
+      for (int i = 0; i < n + 2; ++i) {
+        const int slot = np % WG_NS;
+        const int lo = i < 2 ? 0 : i - 2, hi = i < n ? i : n - 1;
+        if (!mbar_wait(s_full + 8 * slot, (uint32_t)(np / WG_NS & 1), polls)) { ok = false; break; }
+        tc_fence_after();
+        const int blk = (no + lo) % WG_R, nb = hi - lo + 1, b0 = lo - (i - 2);
+        const int n1 = blk + nb > WG_R ? WG_R - blk : nb;
+        const uint64_t ad0 = umma_desc(s0 + slot * WG_A, WG_ROW, WG_CH);
+        const uint64_t bd0 = umma_desc(s_dz, WG_DROW, U_TX * 16);
+        auto mma = [&](int kx, int rp, int blk0, int cnt, int off) {
           asm volatile(
               "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (uint32_t)(acc * C)),
-              "l"(ad), "l"(bd), "r"(kIdescWgrad), "r"(accum)
+              "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem + (uint32_t)(kx * WG_N + off * C)),
+              "l"(ad0 + (uint64_t)(2 * rp * (WG_ROW / 16) + kx)),
+              "l"(bd0 + (uint64_t)(2 * rp * (WG_DROW / 16) + blk0 * (4 * U_TX))), "r"(idesc_wgrad(cnt * C)), "r"(1u)
               : "memory");
+        };
+#pragma unroll 1
+        for (int kx = 0; kx < 3; ++kx) {
+#pragma unroll
+          for (int rp = 0; rp < U_TY / 2; ++rp) {
+            mma(kx, rp, blk, n1, b0);
+            if (n1 < nb) mma(kx, rp, 0, nb - n1, b0 + n1);
+          }
         }
+        tc_commit(s_free + 8 * slot);
+        ++np;
       }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s_done + 8 * s)
-                   : "memory");
-      // refill the stage of the previous tile once its MMAs and warp 1 are done with it
-      if (it >= 1 && it - 1 + WG_NS < nmine) {
-        const int sp = (it - 1) % WG_NS;
-        const uint32_t pp = (uint32_t)((it - 1) / WG_NS) & 1u;
-        if (!mbar_wait(s_done + 8 * sp, pp, polls) || !mbar_wait(s_freed + 8 * sp, pp, polls)) { ok = false; break; }
-        int x0, y0, z0;
-        origin(blockIdx.x + (it - 1 + WG_NS) * gridDim.x, x0, y0, z0);
-        wg_issue(maps, s0 + sp * WG_STAGE, s_full + 8 * sp, x0, y0, z0);
-        odd ^= 1u << sp;
+      no += n;
+    }
+    if (lane == 0) tc_commit(s_fin);
+    __syncwarp();
+  } else if (warp < 4) {
+    // ---------------- bias gradient: this thread's chunk c = tid & 3 ... of voxels tid / 4 + 32 q
+    const unsigned char* base = smem + (s_dz - smem_u32(smem));
+    const int c = threadIdx.x & 3, v0 = threadIdx.x >> 2;
+    int np = 0, no = 0;
+    while (ok && runs.next(d.nz, col, za, zb)) {
+      const int n = zb - za;
+      for (int i = 0; i < n + 2; ++i) {
+        const int slot = np % WG_NS;
+        if (!mbar_wait(s_full + 8 * slot, (uint32_t)(np / WG_NS & 1), polls)) { ok = false; break; }
+        if (i < n) {
+          const unsigned char* t = base + ((no + i) % WG_R) * (4 * U_TX * 16) + c * U_TX * 16;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int v = v0 + 32 * q;
+            float f[8];
+            unpack8(*reinterpret_cast<const uint4*>(t + (v >> 3) * WG_DROW + (v & 7) * 16), f);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) bacc[e] += f[e];
+          }
+        }
+        mbar_arrive(s_free + 8 * slot);
+        ++np;
       }
+      no += n;
     }
-    // every MMA issued so far, then the copies still in flight (only after a timeout)
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(s_fin) : "memory");
-    if (!ok)
-      for (int b = 0; b < WG_NS; ++b)
-        if ((used >> b) & 1u) mbar_drain(s_full + 8 * b, ((odd >> b) & 1u) ^ 1u);
-  } else if (warp == 1) {
-    // bias gradient: bacc = sum of dz[p][co = lane] over this CTA's voxels
-    for (int it = 0; it < nmine && ok; ++it) {
-      const int s = it % WG_NS;
-      const uint32_t ph = (uint32_t)(it / WG_NS) & 1u;
-      if (!mbar_wait(s_full + 8 * s, ph, polls)) { ok = false; break; }
-      const unsigned char* b = smem + (s0 - smem_u32(smem)) + s * WG_STAGE + WG_A;
-      const int c = lane >> 3, e = lane & 7;
-#pragma unroll 8
-      for (int v = 0; v < U_TY * U_TX; ++v)
-        bacc += __bfloat162float(*reinterpret_cast<const bf16*>(b + ((v >> 3) * 4 + c) * 128 + (v & 7) * 16 + e * 2));
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(s_freed + 8 * s) : "memory");
-    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) s_b[threadIdx.x * 8 + e] = bacc[e];
   }
   const bool fin = mbar_drain(s_fin, 0);   // every MMA issued, also after a give-up: TMEM is freed below
   if (__syncthreads_or(!ok || !fin)) {
@@ -741,10 +798,10 @@ k_wgrad_tc05(const __grid_constant__ WgradMaps maps, float* __restrict__ part, f
   } else {
     tc_fence_after();
     if (warp < 3) {
-      // lane = ci, TMEM lanes 32 ky .. 32 ky + 31; accumulator (kz, kx) -> tap kz*9 + ky*3 + kx
+      // lane = ci, TMEM lanes 32 ky .. 32 ky + 31; columns kx * 96 + (2 - kz) * 32 + co
 #pragma unroll 1
-      for (int q = 0; q < 18; ++q) {            // accumulator q / 2, columns (co) 16 (q % 2) .. + 15
-        const int acc = q >> 1, co0 = (q & 1) * 16;
+      for (int q = 0; q < 18; ++q) {            // (kx, 2 - kz) = q / 2, columns (co) 16 (q % 2) .. + 15
+        const int acc = q >> 1, co0 = (q & 1) * 16, kx = acc / 3, kz = 2 - acc % 3;
         uint32_t r[16];
         asm volatile(
             "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
@@ -752,13 +809,16 @@ k_wgrad_tc05(const __grid_constant__ WgradMaps maps, float* __restrict__ part, f
               "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
             : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * C + co0)));
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const int tap = (acc / 3) * 9 + warp * 3 + acc % 3;
+        const int tap = kz * 9 + warp * 3 + kx;
         float* pp = part + ((size_t)blockIdx.x * NTAP + tap) * (C * C) + co0 * C + lane;
 #pragma unroll
         for (int j = 0; j < 16; ++j) pp[j * C] = __uint_as_float(r[j]);
       }
+    } else if (warp == 3 && bpart) {
+      float t = 0.f;                            // feature lane: chunk lane / 8, the 32 threads of that chunk
+      for (int v = 0; v < 32; ++v) t += s_b[(v * 4 + (lane >> 3)) * 8 + (lane & 7)];
+      bpart[(size_t)blockIdx.x * C + lane] = t;
     }
-    if (warp == 1 && bpart) bpart[(size_t)blockIdx.x * C + lane] = bacc;
   }
   tc_fence_before();
   __syncthreads();
@@ -997,16 +1057,41 @@ k_wgrad_last(const float* __restrict__ d6, const bf16* __restrict__ a5, float* _
 
 // ------------------------------------------------------------------ reductions, input, parameters
 
-enum { MAP_PLAIN = 0, MAP_MID = 1, MAP_FIRST = 2, MAP_LAST = 3 };
+enum { MAP_MID = 1, MAP_FIRST = 2, MAP_LAST = 3 };
 
-// out[map(i)] = sum_b part[b*n + i] (fixed order, double accumulation).
+// sum_b p[b * n], b = 0 .. P-1, in that order, eight loads in flight: the loop
+// is one load latency per trip (a 31x120x100 layer's weight gradient took 99.7
+// us with four loads a trip and blocks of 256, 79.5 so, in blocks of 64 and
+// with the biases in the same launch).
+__device__ __forceinline__ double sum_parts(const float* __restrict__ p, int P, size_t n) {
+  double s = 0.0;
+  int b = 0;
+  for (; b + 8 <= P; b += 8) {
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = p[(size_t)(b + e) * n];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) s += v[e];
+  }
+  for (; b < P; ++b) s += p[(size_t)b * n];
+  return s;
+}
+
+constexpr int kReduceThreads = 64;
+
+// out[map(i)] = sum_b part[b*n + i] (fixed order, double accumulation), and with bout the C biases
+// bout[c] = sum_b bpart[b*C + c].
 // MAP_MID: i = (tap*32 + co)*32 + ci -> (co*32 + ci)*27 + tap; MAP_FIRST:
 // i = tap*32 + co -> co*27 + tap; MAP_LAST: i = (tap*32 + ci)*K + k -> (k*32 + ci)*27 + tap.
-__global__ void k_reduce_part(const float* __restrict__ part, int P, int n, float* __restrict__ out, int map, int K) {
+__global__ void __launch_bounds__(kReduceThreads)
+k_reduce_part(const float* __restrict__ part, int P, int n, float* __restrict__ out, int map, int K,
+              const float* __restrict__ bpart, float* __restrict__ bout) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double s = 0.0;
-  for (int b = 0; b < P; ++b) s += part[(size_t)b * n + i];
+  if (i >= n) {
+    if (bout && i - n < C) bout[i - n] = (float)sum_parts(bpart + (i - n), P, C);
+    return;
+  }
+  const double s = sum_parts(part + i, P, n);
   int j = i;
   if (map == MAP_MID) {
     const int t = i >> 10, co = (i >> 5) & 31, ci = i & 31;
@@ -1227,35 +1312,6 @@ cudaError_t configure_once(int K) {
 }
 
 // Launch helpers (all persistent: grids bounded by the tile count).
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
-
-// A host-side failure of a layer launch (a tensor map that could not be
-// encoded), reported by the next status check of the calling entry point.
-cudaError_t g_launch_err = cudaSuccess;
-
-cudaError_t take_launch_error() {
-  const cudaError_t e = g_launch_err;
-  g_launch_err = cudaSuccess;
-  return e != cudaSuccess ? e : cudaGetLastError();
-}
-
 // Tiles of 128 voxels and the persistent grid of k_conv_tc05 (two CTAs per SM).
 int tc05_tiles(const Dims& d, int& tx, int& ty) {
   tx = (d.nx + U_TX - 1) / U_TX;
@@ -1286,51 +1342,23 @@ cudaError_t launch_conv(int epi, const bf16* in, const bf16* wk, const float* bi
   return launch_tc05<EPI_MASK>(in, wk, bias, mask, out, d, sms, st, none);
 }
 
-// The two 5-D tensor maps of k_wgrad_tc05 over [z][y][x][32] bfloat16 maps.
-cudaError_t wgrad_maps(const bf16* a, const bf16* dz, const Dims& d, WgradMaps* maps) {
-  EncodeTiledFn enc = encode_tiled();
-  if (!enc) return cudaErrorNotSupported;
-  const cuuint64_t row = (cuuint64_t)C * 2, line = row * d.nx, plane = line * d.ny;
-  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  {
-    const cuuint64_t dims[5] = {8, (cuuint64_t)d.nx, (cuuint64_t)d.nz, 4, (cuuint64_t)d.ny};
-    const cuuint64_t strides[4] = {row, plane, 16, line};
-    const cuuint32_t box[5] = {8, U_HX, 3, 4, WG_HY};
-    if (enc(&maps->a, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)a, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
-  }
-  {
-    const cuuint64_t dims[5] = {8, (cuuint64_t)d.nx, 4, (cuuint64_t)d.ny, (cuuint64_t)d.nz};
-    const cuuint64_t strides[4] = {row, 16, line, plane};
-    const cuuint32_t box[5] = {8, U_TX, 4, U_TY, 1};
-    if (enc(&maps->dz, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)dz, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
-  }
-  return cudaSuccess;
+void launch_reduce(const float* part, int P, int n, float* out, int map, int K, const float* bpart, float* bout,
+                   cudaStream_t st) {
+  k_reduce_part<<<(n + (bout ? C : 0) + kReduceThreads - 1) / kReduceThreads, kReduceThreads, 0, st>>>(
+      part, P, n, out, map, K, bpart, bout);
 }
 
 // Weight and bias gradients of a 32 -> 32 layer: per-CTA partial sums (one
 // CTA per SM, at most part_slots(d) of them), then fixed-order reductions.
 void launch_wgrad_mid(const bf16* a, const bf16* dz, float* part, float* bpart, float* dw, float* db, const Dims& d,
                       int sms, cudaStream_t st) {
-  WgradMaps maps;
-  const cudaError_t e = wgrad_maps(a, dz, d, &maps);
-  if (e != cudaSuccess) {
-    g_launch_err = e;
-    return;
-  }
   int tx, ty;
   const int ntiles = tc05_tiles(d, tx, ty);
   int P = part_slots(d);
   if (P > sms) P = sms;
   if (P > ntiles) P = ntiles;
-  k_wgrad_tc05<<<P, 128, wgrad05_smem, st>>>(maps, part, bpart, d, tx, ty, ntiles);
-  k_reduce_part<<<(WMID + 255) / 256, 256, 0, st>>>(part, P, WMID, dw, MAP_MID, 1);
-  if (db) k_reduce_part<<<1, 32, 0, st>>>(bpart, P, C, db, MAP_PLAIN, 1);
+  k_wgrad_tc05<<<P, 288, wgrad05_smem, st>>>(a, dz, part, bpart, d, tx, ty);
+  launch_reduce(part, P, WMID, dw, MAP_MID, 1, bpart, db, st);
 }
 
 }  // namespace mnet
@@ -1420,7 +1448,7 @@ int fail(muffin_net* n, int code, const std::string& msg) {
 }
 
 int cuda_check(muffin_net* n, const char* what) {
-  const cudaError_t e = take_launch_error();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(n, MUFFIN_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
   return MUFFIN_OK;
 }
@@ -1478,8 +1506,7 @@ void last_train(muffin_net* n, const float* tx, const bf16* taux, bf16* g5) {
   int P = part_slots(d);
   if (P > 2 * n->sms) P = 2 * n->sms;
   k_wgrad_last<K><<<P, 288, wgrad_last_smem(K), n->st>>>(n->d6, a5, n->part, d);
-  k_reduce_part<<<(NTAP * C * K + 255) / 256, 256, 0, n->st>>>(n->part, P, NTAP * C * K, n->grad + w_offset(5),
-                                                               MAP_LAST, K);
+  launch_reduce(n->part, P, NTAP * C * K, n->grad + w_offset(5), MAP_LAST, K, nullptr, nullptr, n->st);
   const int gsimt = d.ntiles < 4 * n->sms ? d.ntiles : 4 * n->sms;
   k_last_bwd_data<K><<<gsimt, 256, last_bwd_smem(K), n->st>>>(n->d6, n->kw.w6b, a5, g5, d);
 }
@@ -1501,8 +1528,7 @@ void loss_and_grad(muffin_net* n, const float* y, const float* tx, const bf16* t
   int P = part_slots(d);
   if (P > 2 * n->sms) P = 2 * n->sms;
   k_wgrad_first<<<P, 288, 0, n->st>>>(n->a0, g, n->part, n->bpart, d);
-  k_reduce_part<<<(NTAP * C + 255) / 256, 256, 0, n->st>>>(n->part, P, NTAP * C, n->grad + w_offset(0), MAP_FIRST, 1);
-  k_reduce_part<<<1, 32, 0, n->st>>>(n->bpart, P, C, n->grad + b_offset(0, n->K), MAP_PLAIN, 1);
+  launch_reduce(n->part, P, NTAP * C, n->grad + w_offset(0), MAP_FIRST, 1, n->bpart, n->grad + b_offset(0, n->K), n->st);
 }
 
 void unpack_params(muffin_net* n) {
@@ -1689,7 +1715,7 @@ static int conv_fail(int code, const std::string& msg) {
 }
 
 static int conv_cuda(const char* what) {
-  const cudaError_t e = take_launch_error();
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return conv_fail(MUFFIN_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
   return MUFFIN_OK;
 }
