@@ -6,13 +6,10 @@
 //
 // Feature maps are [nz][ny][nx][32] bfloat16 (64 bytes per voxel).  The
 // tensor-core kernels (below) march tiles of 1 x 16 x 8 voxels along the
-// channel axis.  The CUDA-core kernels work on output tiles of 2 x 8 x 16
-// voxels (channel, row, column) whose inputs, with a one-voxel halo
-// (4 x 10 x 18), are staged in shared memory by cp.async with zero fill
-// outside the cube (the zero padding of the layers); there a voxel's 64 bytes
-// are four 16-byte chunks, chunk c of row r stored at chunk c ^ ((r >> 1) & 3),
-// so that eight consecutive rows read at the same chunk hit eight different
-// bank groups.
+// channel axis.  The CUDA-core kernels of the 1 -> 32 layer work on output tiles
+// of 2 x 8 x 16 voxels (channel, row, column) whose scalar inputs, with a
+// one-voxel halo (4 x 10 x 18, zero outside the cube: the zero padding of the
+// layers), are staged in shared memory.
 //
 // The 32 -> 32 layers are implicit GEMMs on the tensor cores, bfloat16 in,
 // float32 accumulate:
@@ -25,11 +22,11 @@
 //                 (M = (row offset, ci), N = (channel offset, co), K = voxels), tcgen05.mma
 //                 with the accumulators resident in tensor memory for the CTA's whole run.
 // The last layer's forward (prediction, or the loss and its gradient d6) is
-// the same tcgen05 kernel with N = 16 (weights of maps K .. 15 zero).  The
-// 1 -> 32 layer and the last layer's gradients (27 or 864 multiply-adds per
-// voxel and output, with float32 d6) run on the CUDA cores.  Every reduction
-// over voxels is a per-block partial sum followed by a fixed-order sum:
-// results do not depend on scheduling.
+// the forward kernel with 16 columns an output (weights of maps K .. 15 zero);
+// its gradients are the 32 -> 32 kernels on d6 split into bfloat16 parts
+// (split3).  The 1 -> 32 layer (27 multiply-adds per voxel and output) runs on
+// the CUDA cores.  Every reduction over voxels is a per-block partial sum
+// followed by a fixed-order sum: results do not depend on scheduling.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -81,10 +78,6 @@ inline Dims make_dims(int nz, int ny, int nx) {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ uint32_t swz(int row, int chunk) {
-  return (uint32_t)(row * ROWB + ((chunk ^ ((row >> 1) & 3)) << 4));
-}
-
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int src_bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
@@ -107,22 +100,6 @@ __device__ __forceinline__ bool inside(const Dims& d, int z, int y, int x) {
 
 __device__ __forceinline__ size_t vox(const Dims& d, int z, int y, int x) {
   return ((size_t)z * d.ny + y) * d.nx + x;
-}
-
-// NZS slices of a map starting at channel zs, rows y0-1 .. y0+TY, columns
-// x0-1 .. x0+TX, into swizzled shared rows h = (hz*HY + hy)*HX + hx.
-template <int NZS>
-__device__ __forceinline__ void load_map_halo(uint32_t s, const bf16* __restrict__ g, const Dims& d, int zs, int y0,
-                                              int x0) {
-  constexpr int N = NZS * HY * HX * 4;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    const int c = i & 3, h = i >> 2;
-    const int hx = h % HX, t = h / HX, hy = t % HY, hz = t / HY;
-    const int gz = zs + hz, gy = y0 - 1 + hy, gx = x0 - 1 + hx;
-    const bool ok = inside(d, gz, gy, gx);
-    const bf16* src = ok ? g + vox(d, gz, gy, gx) * C + c * 8 : g;
-    cp_async16(s + swz(h, c), src, ok ? 16 : 0);
-  }
 }
 
 // Scalar field halo (float32 cube or bfloat16 single-feature map) into s[h], zero outside.
@@ -174,10 +151,39 @@ struct LastArgs {
   const float* s;             // input scale (device scalar)
   const float* tx;            // EPI_LOSS: target cube [V]
   const bf16* taux;           // EPI_LOSS: target fields [nz][K-1][ny][nx]
-  float* d6;                  // EPI_LOSS: loss gradient [V][K]
+  bf16* d6;                   // EPI_LOSS: loss gradient [V][32], split in three (split3)
   double* lpart;              // EPI_LOSS: per-CTA partial sums [grid][K+1]
   float* out_x;               // EPI_PRED: cube [V]
   float* out_aux;             // EPI_PRED: fields [nz][K-1][ny][nx]
+};
+
+// The loss gradient of the last layer is float32.  It goes to the tensor cores
+// as three bfloat16 values that add up to it exactly, hi + mid + lo (8 bits of
+// its significand each), in a map of 32 features: map k's parts in features k,
+// 8 + k and 16 + k.  Its products with bfloat16 weights and maps are exact in
+// float32, so the two gradients of the last layer are the 32 -> 32 kernels.
+constexpr int kSplit = 8;                    // features between the parts
+__device__ __forceinline__ void split3(float v, float& hi, float& mid, float& lo) {
+  hi = __uint_as_float(__float_as_uint(v) & 0xffff0000u);
+  mid = lo = 0.f;
+  if (!(fabsf(v) <= 3.402823466e38f)) {      // infinity or NaN
+    hi = v;
+    return;
+  }
+  const float r = v - hi;
+  mid = __uint_as_float(__float_as_uint(r) & 0xffff0000u);
+  lo = r - mid;
+}
+
+// Sum of floats in two floats (Knuth's two-sum), for the few terms between two
+// additions to a double: double arithmetic runs at 1/64 of the float rate.
+struct Pair {
+  float hi, lo;
+  __device__ __forceinline__ void add(float x, float e) {
+    const float t = hi + x, b = t - hi;
+    lo += ((hi - (t - b)) + (x - b)) + e;
+    hi = t;
+  }
 };
 
 // ------------------------------------------------------------------ 32 -> 32 layers on tcgen05 (UMMA), marching along z
@@ -351,10 +357,18 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
   Runs runs(tiles_x * tiles_y, d.nz);
   int col, za, zb;
   bool ok = true;
-  double l2 = 0.0;
-  double lsum[kMaxOut];
+  // EPI_LOSS: sums of up to eight tiles (lam r^2, then r of each map), and per thread the doubles they go to
+  __shared__ double s_loss[EPI == EPI_LOSS ? (kMaxOut + 1) * 128 : 1];
+  double* tsum = s_loss + (EPI == EPI_LOSS ? threadIdx.x & 127 : 0);
+  Pair psum[EPI == EPI_LOSS ? kMaxOut + 1 : 1];
+  auto flush = [&] {
 #pragma unroll
-  for (int k = 0; k < kMaxOut; ++k) lsum[k] = 0.0;
+    for (int k = 0; k <= kMaxOut; ++k) {
+      if (k > la.K) break;
+      tsum[128 * k] += (double)psum[k].hi + (double)psum[k].lo;
+      psum[k] = Pair{0.f, 0.f};
+    }
+  };
 
   if (warp >= 4 && warp < 8) {
     // ---------------- loaders: planes za-1 .. zb of each stretch, two planes in flight behind the newest
@@ -462,10 +476,19 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
     float bn[NO];
 #pragma unroll
     for (int c = 0; c < NO; ++c) bn[c] = (EPI != EPI_MASK && bias && (!kLast || c < la.K)) ? bias[c] : 0.f;
-    // last layer: input scale
+    // last layer: input scale; factors of the loss gradient
     const float sc = kLast ? *la.s : 1.f;
     const float inv_sc = 1.0f / sc;
-    const double gs = 2.0 / (double)d.nvox;
+    float gk[EPI == EPI_LOSS ? kMaxOut : 1];
+    if constexpr (EPI == EPI_LOSS) {
+#pragma unroll
+      for (int k = 0; k < kMaxOut; ++k) gk[k] = (float)(2.0 / (double)d.nvox * la.lam.v[k]);
+#pragma unroll
+      for (int k = 0; k <= kMaxOut; ++k) {
+        tsum[128 * k] = 0.0;
+        psum[k] = Pair{0.f, 0.f};
+      }
+    }
     const size_t plane = (size_t)d.ny * d.nx;
     const int m = warp * 32 + lane;
     int no = 0;
@@ -473,6 +496,17 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
       const int x = (col % tiles_x) * U_TX + (m & 7), y = (col / tiles_x) * U_TY + (m >> 3);
       for (int z = za; z < zb; ++z, ++no) {
         const int acc = no % Z_RING;
+        // the loss's targets, loaded while the tile's MMAs run
+        float tk[EPI == EPI_LOSS ? kMaxOut : 1];
+        if constexpr (EPI == EPI_LOSS) {
+          if (inside(d, z, y, x)) {
+            tk[0] = la.tx[vox(d, z, y, x)];
+            const bf16* ta = la.taux + (size_t)z * (la.K - 1) * plane + (size_t)y * d.nx + x;
+#pragma unroll
+            for (int k = 1; k < kMaxOut; ++k)
+              if (k < la.K) tk[k] = __bfloat162float(ta[(size_t)(k - 1) * plane]);
+          }
+        }
         if (!mbar_wait(s_done + 8 * acc, (uint32_t)(no / Z_RING & 1), polls)) { ok = false; break; }
         tc_fence_after();
         const uint32_t taddr = tmem + (uint32_t)(acc * NO) + ((uint32_t)(warp * 32) << 16);
@@ -528,30 +562,42 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           tc_fence_before();
           mbar_arrive(s_read + 8 * acc);
-          if (inside(d, z, y, x)) {
+            if (inside(d, z, y, x)) {
             const int K = la.K;
             const size_t v = vox(d, z, y, x);
             const size_t a0 = ((size_t)z * (K > 1 ? K - 1 : 1)) * plane + (size_t)y * d.nx + x;
-    #pragma unroll
+            float part[EPI == EPI_LOSS ? 3 * kSplit : 1] = {};
+#pragma unroll
             for (int k = 0; k < kMaxOut; ++k) {
               if (k < K) {
                 const float zk = __uint_as_float(r[k]) + bn[k];
                 if constexpr (EPI == EPI_LOSS) {
-                  const float tk = k == 0 ? la.tx[v] * inv_sc : __bfloat162float(la.taux[a0 + (size_t)(k - 1) * plane]);
-                  const float rk = zk - tk;
-                  la.d6[v * K + k] = (float)(gs * la.lam.v[k]) * rk;
-                  l2 += (double)la.lam.v[k] * rk * rk;
-                  lsum[k] += rk;
+                  const float rk = zk - (k == 0 ? tk[0] * inv_sc : tk[k]), lk = la.lam.v[k];
+                  split3(gk[k] * rk, part[k], part[kSplit + k], part[2 * kSplit + k]);
+                  // lam r^2 and r with their rounding errors where those are float32 values, else in double
+                  const float p = lk * rk, q = p * rk;
+                  if (q >= 1e-28f && q <= 1e30f) psum[0].add(q, fmaf(p, rk, -q) + fmaf(lk, rk, -p) * rk);
+                  else tsum[0] += (double)lk * rk * rk;
+                  if (fabsf(rk) <= 1e30f) psum[k + 1].add(rk, 0.f);
+                  else tsum[128 * (k + 1)] += rk;
                 } else {
                   if (k == 0) la.out_x[v] = fmaxf(sc * zk, 0.f);
                   else la.out_aux[a0 + (size_t)(k - 1) * plane] = fminf(fmaxf(zk, -1.f), 1.f);
                 }
               }
             }
+            if constexpr (EPI == EPI_LOSS) {
+              uint4* o = reinterpret_cast<uint4*>(la.d6 + v * C);
+#pragma unroll
+              for (int q = 0; q < 3; ++q) o[q] = pack8(part + 8 * q);
+              o[3] = make_uint4(0u, 0u, 0u, 0u);
+            }
           }
+          if (EPI == EPI_LOSS && (no & 7) == 7) flush();
         }
       }
     }
+    if (EPI == EPI_LOSS) flush();
   }
   const bool fin = mbar_drain(s_fin, 0);   // every copy and MMA issued, also after a give-up: TMEM is freed below
   tc_fence_before();
@@ -560,14 +606,10 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
   if constexpr (EPI == EPI_LOSS) {
     // lpart[block] = (sum_k lam_k sum_p r_k^2, sum_p r_0, ..., sum_p r_{K-1}), fixed order
-    const double t2 = muffin::block_sum(l2, s_red);
-    if (threadIdx.x == 0) la.lpart[(size_t)blockIdx.x * (la.K + 1)] = t2;
-#pragma unroll
-    for (int k = 0; k < kMaxOut; ++k) {
-      if (k >= la.K) break;
+    for (int k = 0; k <= la.K; ++k) {
+      const double t = muffin::block_sum(threadIdx.x < 128 ? tsum[128 * k] : 0.0, s_red);
+      if (threadIdx.x == 0) la.lpart[(size_t)blockIdx.x * (la.K + 1) + k] = t;
       __syncthreads();
-      const double tk = muffin::block_sum(lsum[k], s_red);
-      if (threadIdx.x == 0) la.lpart[(size_t)blockIdx.x * (la.K + 1) + 1 + k] = tk;
     }
   }
 }
@@ -581,8 +623,13 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
 // 128 x 96 per kx holds the nine row and channel offsets of its taps (rows
 // 96..127, "ky = 3", are computed and dropped).  The three accumulators (288
 // columns) stay in tensor memory for the CTA's whole run over its tiles; the
-// sums leave TMEM once, at the end.  24 MMAs of N = 96 per tile replace 72 of
-// N = 32; an MMA takes as long either way (the read of its A operand).
+// sums leave TMEM once, at the end, or every `flush` planes: the tensor core
+// adds with truncation, which over a run of 1700 additions of one sign costs
+// 1e-4 of the sum.  The 32 -> 32 layers' bfloat16 gradients carry that anyway;
+// the last layer's, whose operand is exact (split3), is flushed every 4 planes
+// (32 additions) onto float32 sums in shared memory, rounded to nearest.  24 MMAs of N = 96 per
+// tile replace 72 of N = 32; an MMA takes as long either way (the read of its A
+// operand).
 //
 // Both operands are MN-major (M or N contiguous: the 8 features of a chunk),
 // canonical layout without swizzle: core matrices of 8 voxels x 16 bytes.  A
@@ -608,9 +655,12 @@ constexpr int WG_R = 8;                                // ring of dz tiles (more
 constexpr int WG_DROW = WG_R * 4 * U_TX * 16;          // row pitch of the ring 4096 B
 constexpr int WG_B = U_TY * WG_DROW;                   // 65536 B
 constexpr int WG_BAR = WG_NS * WG_A + WG_B;            // full, free, fin, TMEM slot
-constexpr int wgrad05_smem = 120 * 1024;               // more than half an SM: one CTA holds all of the tensor memory
-static_assert(WG_BAR + 256 + 128 <= wgrad05_smem, "weight gradient shared memory");
+constexpr int WG_SUM = 3 * 3 * C * 96 * 4;              // flushed sums, 110592 B
+// more than half an SM in any case: one CTA holds all of the tensor memory
+__host__ __device__ constexpr int wgrad05_smem(bool flush) { return flush ? WG_BAR + 256 + 128 + WG_SUM : 120 * 1024; }
+static_assert(WG_BAR + 256 + 128 <= wgrad05_smem(false) && wgrad05_smem(true) + 4096 <= muffin::kMaxDynSmem, "weight gradient shared memory");
 constexpr int WG_N = 3 * C;
+constexpr int kLastFlush = 4;                          // planes between two flushes, last layer
 // D f32, A/B bf16, both MN-major, N = n, M = 128
 __host__ __device__ constexpr uint32_t idesc_wgrad(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) |
@@ -619,7 +669,7 @@ __host__ __device__ constexpr uint32_t idesc_wgrad(int n) {
 
 __global__ void __launch_bounds__(288, 1)
 k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __restrict__ part,
-             float* __restrict__ bpart, Dims d, int tiles_x, int tiles_y) {
+             float* __restrict__ bpart, Dims d, int tiles_x, int tiles_y, int flush) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ float s_b[128 * 8];
   const uint32_t s0 = (smem_u32(smem) + 127u) & ~127u;
@@ -627,7 +677,9 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
   const uint32_t s_full = s0 + WG_BAR;          // plane and dz tile loaded, per slot (128 loader threads)
   const uint32_t s_free = s_full + 8 * WG_NS;   // MMAs done and dz summed, per slot (1 + 128 threads)
   const uint32_t s_fin = s_free + 8 * WG_NS;    // every MMA of the CTA finished
-  const uint32_t s_tm = s_fin + 8;
+  const uint32_t s_stop = s_fin + 8;            // MMAs before a flush finished
+  const uint32_t s_go = s_stop + 8;             // accumulators stored and cleared (96 threads)
+  const uint32_t s_tm = s_go + 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int b = 0; b < WG_NS; ++b) {
@@ -635,6 +687,8 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
       muffin::mbar_init(s_free + 8 * b, 129);
     }
     muffin::mbar_init(s_fin, 1);
+    muffin::mbar_init(s_stop, 1);
+    muffin::mbar_init(s_go, 96);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -646,14 +700,43 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
   tc_fence_after();
   uint32_t tmem;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(s_tm) : "memory");
-  if (warp < 4) {                               // accumulators start at zero
+  auto clear = [&] {                            // warps 0-3: this warp's lanes of the accumulators
     const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16);
     for (int c = 0; c < 3 * WG_N; c += 8)
       asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(ta + (uint32_t)c),
                    "r"(0u)
                    : "memory");
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-  }
+  };
+  // warps 0-2: the sums out of tensor memory, onto this CTA's flushed sums (s_sum, flush > 0), and at the end to part
+  float* s_sum = reinterpret_cast<float*>(smem + (s0 - smem_u32(smem)) + WG_BAR + 256);
+  auto store = [&](bool add, bool last) {
+    // lane = ci, TMEM lanes 32 ky .. 32 ky + 31; columns kx * 96 + (2 - kz) * 32 + co
+#pragma unroll 1
+    for (int q = 0; q < 18; ++q) {            // (kx, 2 - kz) = q / 2, columns (co) 16 (q % 2) .. + 15
+      const int acc = q >> 1, co0 = (q & 1) * 16, kx = acc / 3, kz = 2 - acc % 3;
+      uint32_t r[16];
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+            "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+          : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * C + co0)));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      float* sp = s_sum + (size_t)(q * 16) * 96 + warp * 32 + lane;
+      float v[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]) + (add ? sp[j * 96] : 0.f);
+      const int tap = kz * 9 + warp * 3 + kx;
+      float* pp = part + ((size_t)blockIdx.x * NTAP + tap) * (C * C) + co0 * C + lane;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        if (last) pp[j * C] = v[j];
+        else sp[j * 96] = v[j];
+      }
+    }
+  };
+  bool flushed = false;
+  if (warp < 4) clear();                        // accumulators start at zero
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -758,6 +841,11 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
         }
         tc_commit(s_free + 8 * slot);
         ++np;
+        if (flush > 0 && np % flush == 0) {
+          tc_commit(s_stop);
+          if (!mbar_wait(s_go, (uint32_t)(np / flush - 1) & 1u, polls)) { ok = false; break; }
+          tc_fence_after();
+        }
       }
       no += n;
     }
@@ -786,6 +874,16 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
         }
         mbar_arrive(s_free + 8 * slot);
         ++np;
+        if (flush > 0 && np % flush == 0 && warp < 3) {
+          const bool stopped = mbar_wait(s_stop, (uint32_t)(np / flush - 1) & 1u, polls);
+          if (!__all_sync(0xffffffffu, stopped)) { ok = false; break; }
+          tc_fence_after();
+          store(flushed, false);
+          flushed = true;
+          clear();
+          tc_fence_before();
+          mbar_arrive(s_go);
+        }
       }
       no += n;
     }
@@ -798,22 +896,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
   } else {
     tc_fence_after();
     if (warp < 3) {
-      // lane = ci, TMEM lanes 32 ky .. 32 ky + 31; columns kx * 96 + (2 - kz) * 32 + co
-#pragma unroll 1
-      for (int q = 0; q < 18; ++q) {            // (kx, 2 - kz) = q / 2, columns (co) 16 (q % 2) .. + 15
-        const int acc = q >> 1, co0 = (q & 1) * 16, kx = acc / 3, kz = 2 - acc % 3;
-        uint32_t r[16];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-              "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-            : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * C + co0)));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        const int tap = kz * 9 + warp * 3 + kx;
-        float* pp = part + ((size_t)blockIdx.x * NTAP + tap) * (C * C) + co0 * C + lane;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) pp[j * C] = __uint_as_float(r[j]);
-      }
+      store(flushed, true);
     } else if (warp == 3 && bpart) {
       float t = 0.f;                            // feature lane: chunk lane / 8, the 32 threads of that chunk
       for (int v = 0; v < 32; ++v) t += s_b[(v * 4 + (lane >> 3)) * 8 + (lane & 7)];
@@ -880,67 +963,6 @@ k_first_fwd(const bf16* __restrict__ a0, const float* __restrict__ w, const floa
   }
 }
 
-// g5[p][ci] = (a5[p][ci] > 0) * sum_tap sum_k d6[p - d(tap)][k] w[tap][k][ci].
-template <int K>
-__global__ void __launch_bounds__(256)
-k_last_bwd_data(const float* __restrict__ d6, const float* __restrict__ w, const bf16* __restrict__ a5,
-                bf16* __restrict__ g5, Dims d) {
-  extern __shared__ __align__(16) float smf[];
-  float* s_w = smf;                      // [27][K][32]
-  float* s_h = smf + NTAP * K * C;       // [HV][K]
-  for (int i = threadIdx.x; i < NTAP * K * C; i += blockDim.x) s_w[i] = w[i];
-  int tz, ty, tx;
-  thread_voxel(tz, ty, tx);
-  for (int tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) {
-    int z0, y0, x0;
-    tile_origin(tile, d, z0, y0, x0);
-    __syncthreads();
-    for (int i = threadIdx.x; i < HV * K; i += blockDim.x) {
-      const int h = i / K, k = i - h * K;
-      const int hx = h % HX, r = h / HX, hy = r % HY, hz = r / HY;
-      const int gz = z0 - 1 + hz, gy = y0 - 1 + hy, gx = x0 - 1 + hx;
-      s_h[i] = inside(d, gz, gy, gx) ? d6[vox(d, gz, gy, gx) * K + k] : 0.f;
-    }
-    __syncthreads();
-    float acc[C];
-#pragma unroll
-    for (int c = 0; c < C; ++c) acc[c] = 0.f;
-#pragma unroll 1
-    for (int t = 0; t < NTAP; ++t) {
-      const int kz = t / 9, ky = (t / 3) % 3, kx = t % 3;
-      const int hh = ((tz + 2 - kz) * HY + ty + 2 - ky) * HX + tx + 2 - kx;
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const float dv = s_h[hh * K + k];
-        const float4* wr = reinterpret_cast<const float4*>(s_w + (t * K + k) * C);
-#pragma unroll
-        for (int q = 0; q < C / 4; ++q) {
-          const float4 wv = wr[q];
-          acc[4 * q] = fmaf(dv, wv.x, acc[4 * q]);
-          acc[4 * q + 1] = fmaf(dv, wv.y, acc[4 * q + 1]);
-          acc[4 * q + 2] = fmaf(dv, wv.z, acc[4 * q + 2]);
-          acc[4 * q + 3] = fmaf(dv, wv.w, acc[4 * q + 3]);
-        }
-      }
-    }
-    const int z = z0 + tz, y = y0 + ty, x = x0 + tx;
-    if (inside(d, z, y, x)) {
-      const size_t v = vox(d, z, y, x);
-      const uint4* m = reinterpret_cast<const uint4*>(a5 + v * C);
-      uint4* o = reinterpret_cast<uint4*>(g5 + v * C);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        float mf[8];
-        unpack8(m[q], mf);
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          if (!(mf[e] > 0.f)) acc[8 * q + e] = 0.f;
-        o[q] = pack8(acc + 8 * q);
-      }
-    }
-  }
-}
-
 // part[b][tap][co] = sum_p g1[p][co] a0[p + d(tap)]; bpart[b][co] = sum_p g1[p][co].
 // 288 threads: thread (kz, ky, co) keeps the three taps kx = 0..2 of its row
 // offset and walks each tile row along x with a sliding window of three a0
@@ -993,68 +1015,6 @@ k_wgrad_first(const bf16* __restrict__ a0, const bf16* __restrict__ g1, float* _
 }
 
 
-// part[b][tap][ci][k] = sum_p d6[p][k] a5[p + d(tap)][ci].  288 threads:
-// thread (kz, ky, ci) keeps the three taps kx = 0..2 of its row offset for
-// all K maps in registers and walks each tile row along x with a sliding
-// window of three a5 values, so that one a5 read and the voxel's K d6 values
-// (read by the whole block at once) feed 3 K multiply-adds.
-template <int K>
-__global__ void __launch_bounds__(288)
-k_wgrad_last(const float* __restrict__ d6, const bf16* __restrict__ a5, float* __restrict__ part, Dims d) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  const uint32_t sa = smem_u32(smem);
-  float* s_d = reinterpret_cast<float*>(smem + HV * ROWB);   // [TV][K]
-  const int ci = threadIdx.x & 31, kzy = threadIdx.x >> 5, kz = kzy / 3, ky = kzy % 3;
-  const unsigned char* a_ci = smem + (ci & 7) * 2;
-  float acc[3][K];
-#pragma unroll
-  for (int kx = 0; kx < 3; ++kx)
-#pragma unroll
-    for (int k = 0; k < K; ++k) acc[kx][k] = 0.f;
-  for (int tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) {
-    int z0, y0, x0;
-    tile_origin(tile, d, z0, y0, x0);
-    __syncthreads();
-    load_map_halo<HZ>(sa, a5, d, z0 - 1, y0, x0);
-    for (int i = threadIdx.x; i < TV * K; i += blockDim.x) {
-      const int r = i / K, k = i - r * K;
-      const int gz = z0 + (r >> 7), gy = y0 + ((r >> 4) & 7), gx = x0 + (r & 15);
-      s_d[i] = inside(d, gz, gy, gx) ? d6[vox(d, gz, gy, gx) * K + k] : 0.f;
-    }
-    cp_async_wait_all();
-    __syncthreads();
-#pragma unroll 1
-    for (int row = 0; row < TZ * TY; ++row) {
-      const int tz = row >> 3, ty = row & 7;
-      const int h0 = ((tz + kz) * HY + ty + ky) * HX;   // halo row of this thread's taps
-      auto av = [&](int hx) {
-        return __bfloat162float(*reinterpret_cast<const bf16*>(a_ci + swz(h0 + hx, ci >> 3)));
-      };
-      float w0 = av(0), w1 = av(1);
-#pragma unroll 4
-      for (int tx = 0; tx < TX; ++tx) {
-        const float w2 = av(tx + 2);
-        const float* dv = s_d + (row * TX + tx) * K;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          const float g = dv[k];
-          acc[0][k] = fmaf(g, w0, acc[0][k]);
-          acc[1][k] = fmaf(g, w1, acc[1][k]);
-          acc[2][k] = fmaf(g, w2, acc[2][k]);
-        }
-        w0 = w1;
-        w1 = w2;
-      }
-    }
-  }
-#pragma unroll
-  for (int kx = 0; kx < 3; ++kx) {
-    float* pp = part + ((size_t)blockIdx.x * (NTAP * C) + (kz * 9 + ky * 3 + kx) * C + ci) * K;
-#pragma unroll
-    for (int k = 0; k < K; ++k) pp[k] = acc[kx][k];
-  }
-}
-
 // ------------------------------------------------------------------ reductions, input, parameters
 
 enum { MAP_MID = 1, MAP_FIRST = 2, MAP_LAST = 3 };
@@ -1082,7 +1042,8 @@ constexpr int kReduceThreads = 64;
 // out[map(i)] = sum_b part[b*n + i] (fixed order, double accumulation), and with bout the C biases
 // bout[c] = sum_b bpart[b*C + c].
 // MAP_MID: i = (tap*32 + co)*32 + ci -> (co*32 + ci)*27 + tap; MAP_FIRST:
-// i = tap*32 + co -> co*27 + tap; MAP_LAST: i = (tap*32 + ci)*K + k -> (k*32 + ci)*27 + tap.
+// i = tap*32 + co -> co*27 + tap; MAP_LAST: i = (tap*K + k)*32 + ci -> (k*32 + ci)*27 + tap, the sum over the three
+// parts of the split loss gradient (features k, 8 + k, 16 + k of a 32 -> 32 weight gradient).
 __global__ void __launch_bounds__(kReduceThreads)
 k_reduce_part(const float* __restrict__ part, int P, int n, float* __restrict__ out, int map, int K,
               const float* __restrict__ bpart, float* __restrict__ bout) {
@@ -1091,17 +1052,22 @@ k_reduce_part(const float* __restrict__ part, int P, int n, float* __restrict__ 
     if (bout && i - n < C) bout[i - n] = (float)sum_parts(bpart + (i - n), P, C);
     return;
   }
-  const double s = sum_parts(part + i, P, n);
   int j = i;
+  double s;
+  if (map == MAP_LAST) {
+    const int ci = i & 31, r = i >> 5, k = r % K, t = r / K;
+    const float* p = part + (t * C + k) * C + ci;
+    s = sum_parts(p, P, WMID) + sum_parts(p + kSplit * C, P, WMID) + sum_parts(p + 2 * kSplit * C, P, WMID);
+    j = (k * C + ci) * NTAP + t;
+  } else {
+    s = sum_parts(part + i, P, n);
+  }
   if (map == MAP_MID) {
     const int t = i >> 10, co = (i >> 5) & 31, ci = i & 31;
     j = (co * C + ci) * NTAP + t;
   } else if (map == MAP_FIRST) {
     const int t = i >> 5, c = i & 31;
     j = c * NTAP + t;
-  } else if (map == MAP_LAST) {
-    const int k = i % K, r = i / K, ci = r & 31, t = r >> 5;
-    j = (k * C + ci) * NTAP + t;
   }
   out[j] = (float)s;
 }
@@ -1113,7 +1079,15 @@ __global__ void k_loss_final(const double* __restrict__ lpart, int P, int K, Lam
   const int k = (int)threadIdx.x - 1;
   if (k >= K) return;
   double acc = 0.0;
-  for (int b = 0; b < P; ++b) acc += lpart[(size_t)b * (K + 1) + 1 + k];
+  int b = 0;
+  for (; b + 8 <= P; b += 8) {      // eight loads in flight, summed in order
+    double v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = lpart[(size_t)(b + e) * (K + 1) + 1 + k];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc += v[e];
+  }
+  for (; b < P; ++b) acc += lpart[(size_t)b * (K + 1) + 1 + k];
   if (k < 0) {
     if (loss) *loss = acc / (double)nvox;
   } else if (grad_b6) {
@@ -1137,12 +1111,13 @@ __global__ void k_maxabs_part(const float* __restrict__ y, long long n, float* _
   }
 }
 
-// s = max |y| (1 if the cube is zero).
+// s = max |y| (1 if the cube is zero).  One warp.
 __global__ void k_scale_final(const float* __restrict__ part, int P, float* __restrict__ s) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   float m = 0.f;
-  for (int b = 0; b < P; ++b) m = fmaxf(m, part[b]);
-  *s = m > 0.f ? m : 1.f;
+  for (int b = threadIdx.x; b < P; b += 32) m = fmaxf(m, part[b]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (threadIdx.x == 0) *s = m > 0.f ? m : 1.f;
 }
 
 // a0 = bf16(y / s).
@@ -1159,8 +1134,7 @@ struct KernelWeights {
   bf16* wf;     // [4][27][32 co][32 ci]   forward operands of layers 2..5
   bf16* wb;     // [4][27][32 ci][32 co]   flipped, transposed: input gradients
   float* bm;    // [4][32]
-  float* w6f;   // [27][32 ci][K]  last layer, forward; bfloat16 values
-  float* w6b;   // [27][K][32 ci]  last layer, input gradient
+  bf16* w6b;    // [27 flipped][32 ci][32]  last layer, input gradient: features k, 8 + k, 16 + k all the weight of map k
   bf16* w6t;    // [27][16 co][32 ci]  last layer, tcgen05 operand (rows K .. 15 zero)
   float* b6;    // [K]
 };
@@ -1196,10 +1170,9 @@ __global__ void k_unpack_params(const float* __restrict__ theta, KernelWeights k
   j -= 4 * LM;
   if (j < K * NTAP * C) {
     const int k = j / (C * NTAP), rem = j % (C * NTAP), ci = rem / NTAP, t = rem % NTAP;
-    const float r = round_bf16(v);
-    kw.w6f[(t * C + ci) * K + k] = r;
-    kw.w6b[(t * K + k) * C + ci] = r;
-    kw.w6t[(t * kLastN + k) * C + ci] = __float2bfloat16_rn(v);
+    const bf16 q = __float2bfloat16_rn(v);
+    for (int p = 0; p < 3; ++p) kw.w6b[((NTAP - 1 - t) * C + ci) * C + p * kSplit + k] = q;
+    kw.w6t[(t * kLastN + k) * C + ci] = q;
   } else {
     kw.b6[j - K * NTAP * C] = v;
   }
@@ -1265,50 +1238,18 @@ int sm_count() {
   return n;
 }
 
-constexpr int last_bwd_smem(int K) { return K * (NTAP * C + HV) * 4; }
-constexpr int wgrad_last_smem(int K) { return HV * ROWB + TV * K * 4; }
-
-template <int K>
-cudaError_t configure_last() {
-  cudaError_t e;
-  if ((e = muffin::allow_max_dyn_smem(k_last_bwd_data<K>)) != cudaSuccess) return e;
-  return muffin::allow_max_dyn_smem(k_wgrad_last<K>);
-}
-
-#define MNET_SWITCH_K(K, EXPR)     \
-  switch (K) {                     \
-    case 1: { constexpr int KK = 1; EXPR; } break; \
-    case 2: { constexpr int KK = 2; EXPR; } break; \
-    case 3: { constexpr int KK = 3; EXPR; } break; \
-    case 4: { constexpr int KK = 4; EXPR; } break; \
-    case 5: { constexpr int KK = 5; EXPR; } break; \
-    case 6: { constexpr int KK = 6; EXPR; } break; \
-    case 7: { constexpr int KK = 7; EXPR; } break; \
-    case 8: { constexpr int KK = 8; EXPR; } break; \
-    default: break;                \
-  }
-
-cudaError_t configure_once(int K) {
-  static bool mid_done = false;
-  static cudaError_t mid_err = cudaSuccess;
-  static bool last_done[kMaxOut + 1] = {};
-  static cudaError_t last_err[kMaxOut + 1] = {};
-  if (!mid_done) {
-    mid_done = true;
-    if ((mid_err = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_RELU>)) == cudaSuccess &&
-        (mid_err = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_BIAS>)) == cudaSuccess &&
-        (mid_err = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_MASK>)) == cudaSuccess &&
-        (mid_err = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_PRED>)) == cudaSuccess &&
-        (mid_err = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_LOSS>)) == cudaSuccess)
-      mid_err = muffin::allow_max_dyn_smem(k_wgrad_tc05);
-  }
-  if (mid_err != cudaSuccess) return mid_err;
-  if (K < 1 || K > kMaxOut) return cudaSuccess;
-  if (!last_done[K]) {
-    last_done[K] = true;
-    MNET_SWITCH_K(K, last_err[K] = configure_last<KK>());
-  }
-  return last_err[K];
+cudaError_t configure_once() {
+  static const cudaError_t err = [] {
+    cudaError_t e;
+    if ((e = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_RELU>)) == cudaSuccess &&
+        (e = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_BIAS>)) == cudaSuccess &&
+        (e = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_MASK>)) == cudaSuccess &&
+        (e = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_PRED>)) == cudaSuccess &&
+        (e = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_LOSS>)) == cudaSuccess)
+      e = muffin::allow_max_dyn_smem(k_wgrad_tc05);
+    return e;
+  }();
+  return err;
 }
 
 // Launch helpers (all persistent: grids bounded by the tile count).
@@ -1348,16 +1289,22 @@ void launch_reduce(const float* part, int P, int n, float* out, int map, int K, 
       part, P, n, out, map, K, bpart, bout);
 }
 
-// Weight and bias gradients of a 32 -> 32 layer: per-CTA partial sums (one
-// CTA per SM, at most part_slots(d) of them), then fixed-order reductions.
-void launch_wgrad_mid(const bf16* a, const bf16* dz, float* part, float* bpart, float* dw, float* db, const Dims& d,
-                      int sms, cudaStream_t st) {
+// Weight (and, with bpart, bias) gradients of a 32 -> 32 layer: per-CTA partial
+// sums, one CTA per SM, at most part_slots(d) of them; returns their number.
+int launch_wgrad_part(const bf16* a, const bf16* dz, float* part, float* bpart, const Dims& d, int flush, int sms,
+                      cudaStream_t st) {
   int tx, ty;
   const int ntiles = tc05_tiles(d, tx, ty);
   int P = part_slots(d);
   if (P > sms) P = sms;
   if (P > ntiles) P = ntiles;
-  k_wgrad_tc05<<<P, 288, wgrad05_smem, st>>>(a, dz, part, bpart, d, tx, ty);
+  k_wgrad_tc05<<<P, 288, wgrad05_smem(flush > 0), st>>>(a, dz, part, bpart, d, tx, ty, flush);
+  return P;
+}
+
+void launch_wgrad_mid(const bf16* a, const bf16* dz, float* part, float* bpart, float* dw, float* db, const Dims& d,
+                      int sms, cudaStream_t st) {
+  const int P = launch_wgrad_part(a, dz, part, bpart, d, 0, sms, st);
   launch_reduce(part, P, WMID, dw, MAP_MID, 1, bpart, db, st);
 }
 
@@ -1391,7 +1338,6 @@ struct muffin_net {
   bf16* act = nullptr;   // training: a1..a5; inference: two ping-pong maps
   bf16* gA = nullptr;
   bf16* gB = nullptr;
-  float* d6 = nullptr;   // [V][K]
 
   bf16* map(int i) const { return act + (size_t)i * d.nvox * C; }
 };
@@ -1418,8 +1364,7 @@ size_t net_layout(muffin_net* n, const Dims& d, int K, int training, char* base)
   kw.wf = (bf16*)take(4 * WMID * 2);
   kw.wb = (bf16*)take(4 * WMID * 2);
   kw.bm = (float*)take(4 * C * 4);
-  kw.w6f = (float*)take(NTAP * C * K * 4);
-  kw.w6b = (float*)take(NTAP * C * K * 4);
+  kw.w6b = (bf16*)take(WMID * 2);
   kw.w6t = (bf16*)take(NTAP * kLastN * C * 2);
   kw.b6 = (float*)take(K * 4);
   float* s = (float*)take(4);
@@ -1433,11 +1378,10 @@ size_t net_layout(muffin_net* n, const Dims& d, int K, int training, char* base)
   bf16* act = (bf16*)take((training ? 5 : 2) * V * C * 2);
   bf16* gA = (bf16*)take(training ? V * C * 2 : 0);
   bf16* gB = (bf16*)take(training ? V * C * 2 : 0);
-  float* d6 = (float*)take(training ? V * K * 4 : 0);
   if (n) {
     n->theta = theta; n->mom1 = m1; n->mom2 = m2; n->grad = grad; n->kw = kw;
     n->s = s; n->mpart = mpart; n->lpart = lpart; n->loss = loss; n->part = part; n->bpart = bpart;
-    n->a0 = a0; n->act = act; n->gA = gA; n->gB = gB; n->d6 = d6;
+    n->a0 = a0; n->act = act; n->gA = gA; n->gB = gB;
   }
   return off;
 }
@@ -1489,26 +1433,23 @@ void last_predict(muffin_net* n, float* x, float* aux) {
   launch_tc05<EPI_PRED>(a5_of(n), n->kw.w6t, n->kw.b6, nullptr, nullptr, n->d, n->sms, n->st, la);
 }
 
-// Last layer of the training pass: loss, d6, its weight and bias gradients,
-// and the gradient of a5's pre-activation into g5.
-template <int K>
-void last_train(muffin_net* n, const float* tx, const bf16* taux, bf16* g5) {
+// Last layer of the training pass: loss, its gradient d6 (into a map, split),
+// the layer's weight and bias gradients, and the gradient of a5's
+// pre-activation into g5.
+void last_train(muffin_net* n, const float* tx, const bf16* taux, bf16* d6, bf16* g5) {
   const Dims& d = n->d;
   bf16* a5 = a5_of(n);
   LastArgs la = last_args(n);
   la.tx = tx;
   la.taux = taux;
-  la.d6 = n->d6;
+  la.d6 = d6;
   la.lpart = n->lpart;
   launch_tc05<EPI_LOSS>(a5, n->kw.w6t, n->kw.b6, nullptr, nullptr, d, n->sms, n->st, la);
-  k_loss_final<<<1, K + 1, 0, n->st>>>(n->lpart, tc05_grid(d, n->sms), K, n->lam, d.nvox, n->loss,
-                                       n->grad + b_offset(5, K));
-  int P = part_slots(d);
-  if (P > 2 * n->sms) P = 2 * n->sms;
-  k_wgrad_last<K><<<P, 288, wgrad_last_smem(K), n->st>>>(n->d6, a5, n->part, d);
-  launch_reduce(n->part, P, NTAP * C * K, n->grad + w_offset(5), MAP_LAST, K, nullptr, nullptr, n->st);
-  const int gsimt = d.ntiles < 4 * n->sms ? d.ntiles : 4 * n->sms;
-  k_last_bwd_data<K><<<gsimt, 256, last_bwd_smem(K), n->st>>>(n->d6, n->kw.w6b, a5, g5, d);
+  k_loss_final<<<1, n->K + 1, 0, n->st>>>(n->lpart, tc05_grid(d, n->sms), n->K, n->lam, d.nvox, n->loss,
+                                          n->grad + b_offset(5, n->K));
+  const int P = launch_wgrad_part(a5, d6, n->part, nullptr, d, kLastFlush, n->sms, n->st);
+  launch_reduce(n->part, P, NTAP * n->K * C, n->grad + w_offset(5), MAP_LAST, n->K, nullptr, nullptr, n->st);
+  launch_conv(EPI_MASK, d6, n->kw.w6b, nullptr, a5, g5, d, n->sms, n->st);
 }
 
 // Loss and gradient into n->grad (training contexts).
@@ -1517,7 +1458,7 @@ void loss_and_grad(muffin_net* n, const float* y, const float* tx, const bf16* t
   forward_to_a5(n, y);
   bf16* g = n->gA;
   bf16* other = n->gB;
-  MNET_SWITCH_K(n->K, last_train<KK>(n, tx, taux, g));
+  last_train(n, tx, taux, other, g);      // `other` holds d6 until the first layer gradient overwrites it
   for (int k = 4; k >= 1; --k) {          // layers 5..2 (index k), input map a_k = map(k - 1)
     const bf16* a_in = n->map(k - 1);
     launch_wgrad_mid(a_in, g, n->part, n->bpart, n->grad + w_offset(k), n->grad + b_offset(k, n->K), d, n->sms,
@@ -1534,6 +1475,7 @@ void loss_and_grad(muffin_net* n, const float* y, const float* tx, const bf16* t
 void unpack_params(muffin_net* n) {
   const int np = param_count(n->K);
   cudaMemsetAsync(n->kw.w6t, 0, NTAP * kLastN * C * 2, n->st);
+  cudaMemsetAsync(n->kw.w6b, 0, WMID * 2, n->st);
   k_unpack_params<<<(np + 255) / 256, 256, 0, n->st>>>(n->theta, n->kw, n->K);
 }
 
@@ -1567,7 +1509,7 @@ int muffin_net_create(muffin_net** out, int nz, int ny, int nx, int n_out, const
   const Dims d = make_dims(nz, ny, nx);
   const size_t need = net_layout(nullptr, d, n_out, training != 0, nullptr);
   if (ws_bytes < need) return MUFFIN_ERR_NOMEM;
-  if (configure_once(n_out) != cudaSuccess) return MUFFIN_ERR_CUDA;
+  if (configure_once() != cudaSuccess) return MUFFIN_ERR_CUDA;
   muffin_net* n = new muffin_net();
   n->training = training != 0;
   n->K = n_out;
@@ -1735,7 +1677,7 @@ static int layer_args(const void* a, const void* b, int nz, int ny, int nx, void
   if (!aligned16(a) || !aligned16(b) || ((uintptr_t)scratch & 255))
     return conv_fail(MUFFIN_ERR_ARG, "maps must be 16-byte aligned, scratch 256-byte aligned");
   if (bytes < muffin_conv3d_scratch_bytes(nz, ny, nx)) return conv_fail(MUFFIN_ERR_NOMEM, "scratch too small");
-  if (configure_once(0) != cudaSuccess) return conv_fail(MUFFIN_ERR_CUDA, "kernel attributes could not be set");
+  if (configure_once() != cudaSuccess) return conv_fail(MUFFIN_ERR_CUDA, "kernel attributes could not be set");
   return MUFFIN_OK;
 }
 
