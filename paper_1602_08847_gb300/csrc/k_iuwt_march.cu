@@ -124,7 +124,8 @@ template <int N, int J1> __device__ __forceinline__ size_t class_at(int gy, int 
 }
 
 // ------------------------------------------------------------------ analysis and spatial dual update
-template <int N, int J1> struct Analysis {
+// LAST: the coarse plane is c_J1 itself (J == J1), its dual U_J is updated here.
+template <int N, int J1, bool LAST> struct Analysis {
   using G = Strip<N, J1>;
   // rows between level 0's input and level j's output
   __host__ __device__ static constexpr int OFF(int j) { return (4 << j) - 2 + j; }
@@ -135,11 +136,11 @@ template <int N, int J1> struct Analysis {
   float* tb;         // vertical sums [2][J1][N]
   int t, y0, y1;
   float k, rho;
-  bool last_dual;    // J == J1: the coarse plane's dual is updated here
 
   RegRing<1> r0;
   RegRing<2> r1;
   float4 x[J1], u[J1];
+  float uc[LAST ? 4 : 1];      // U_J beside u[J1 - 1]
 
   // the rows before the first ones that the steps prefetch, into L2 at once
   __device__ __forceinline__ void ahead() const {
@@ -157,6 +158,13 @@ template <int N, int J1> struct Analysis {
       const int o = e0 + 1 - OFF(j);
       un[j] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (o >= y0 && o < y1) un[j] = ldg4(U + (size_t)j * N * N + (size_t)o * N);
+    }
+    float ucn[LAST ? 4 : 1] = {};
+    if constexpr (LAST) {
+      const int o = e0 + 1 - OFF(J1 - 1);
+      if (o >= y0 && o < y1)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ucn[i] = __ldcg(cls + class_at<N, J1>(o, t, i));
     }
     if ((t & 7) == 0) {
       pf_line(D + (size_t)((e0 + kAheadAn) & (N - 1)) * N);
@@ -187,10 +195,8 @@ template <int N, int J1> struct Analysis {
         if (j == J1 - 1) {
           float v[4] = {cn.x, cn.y, cn.z, cn.w};
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            float* p = cls + class_at<N, J1>(o, t, i);
-            *p = last_dual ? vec::dual1(*p, v[i], k, rho) : v[i];
-          }
+          for (int i = 0; i < 4; ++i)
+            cls[class_at<N, J1>(o, t, i)] = LAST ? vec::dual1(uc[LAST ? i : 0], v[i], k, rho) : v[i];
         }
       }
       if (j + 1 < J1) x[j + 1] = cn;
@@ -198,11 +204,14 @@ template <int N, int J1> struct Analysis {
     x[0] = xn;
 #pragma unroll
     for (int j = 0; j < J1; ++j) u[j] = un[j];
+    if constexpr (LAST)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) uc[i] = ucn[i];
   }
 };
 
 // grid (strips, L); U: [L][J+1][N][N], planes j >= J1 class-permuted
-template <int N, int J1>
+template <int N, int J1, bool LAST>
 __global__ void __launch_bounds__(N / 4, Strip<N, J1>::MINB)
 k_fine_analysis_m(int J, const float* __restrict__ D, float* __restrict__ U, float* __restrict__ cr, float k, float rho,
                   int rows) {
@@ -210,14 +219,13 @@ k_fine_analysis_m(int J, const float* __restrict__ D, float* __restrict__ U, flo
   extern __shared__ __align__(16) float sm[];
   constexpr size_t P = (size_t)N * N;
   const int l = blockIdx.y;
-  Analysis<N, J1> a;
+  Analysis<N, J1, LAST> a;
   a.t = threadIdx.x;
   a.y0 = blockIdx.x * rows;
   a.y1 = min(N, a.y0 + rows);
   a.D = D + (size_t)l * P + 4 * a.t;
   a.U = U + (size_t)l * (J + 1) * P + 4 * a.t;
-  a.last_dual = J == J1;
-  a.cls = J == J1 ? U + ((size_t)l * (J + 1) + J) * P : cr + (size_t)l * P;
+  a.cls = LAST ? U + ((size_t)l * (J + 1) + J) * P : cr + (size_t)l * P;
   a.tb = sm;
   a.ring = sm + 2 * J1 * N + 4 * a.t;
   a.k = k;
@@ -228,6 +236,7 @@ k_fine_analysis_m(int J, const float* __restrict__ D, float* __restrict__ U, flo
 #pragma unroll
   for (int j = 0; j < J1; ++j) a.x[j] = a.u[j] = make_float4(0.f, 0.f, 0.f, 0.f);
   a.x[0] = ldg4(a.D + (size_t)((a.y0 - G::H) & (N - 1)) * N);
+  for (float& v : a.uc) v = 0.f;
 #pragma unroll
   for (int i = 0; i < G::RING; ++i) st4(a.ring + i * N, make_float4(0.f, 0.f, 0.f, 0.f));
   float *lo = a.ring, *hi = a.ring + 8 * N;
@@ -461,9 +470,12 @@ cudaError_t launch_fine_analysis_march(const Geom& g, const IuwtArgs& a, cudaStr
 #define FA(NN, JJ)                                                                                       \
   {                                                                                                      \
     using G = march::Strip<NN, JJ>;                                                                      \
-    const Split p = split_rows(NN, g.L, G::LAG, G::MINB, kAnalysisStep[JJ], false);                                         \
-    march::k_fine_analysis_m<NN, JJ><<<dim3(p.strips, g.L), NN / 4, G::SMEM, s>>>(g.J, a.D, a.U, a.cr, a.k, a.rho, \
-                                                                                  p.rows);               \
+    const Split p = split_rows(NN, g.L, G::LAG, G::MINB, kAnalysisStep[JJ], false);                      \
+    const dim3 grid(p.strips, g.L);                                                                      \
+    if (g.J == JJ)                                                                                       \
+      march::k_fine_analysis_m<NN, JJ, true><<<grid, NN / 4, G::SMEM, s>>>(g.J, a.D, a.U, a.cr, a.k, a.rho, p.rows); \
+    else                                                                                                 \
+      march::k_fine_analysis_m<NN, JJ, false><<<grid, NN / 4, G::SMEM, s>>>(g.J, a.D, a.U, a.cr, a.k, a.rho, p.rows); \
     return cudaGetLastError();                                                                           \
   }
   MARCH_CASES(FA)
@@ -492,7 +504,8 @@ cudaError_t iuwt_march_configure(const Geom& g) {
   if (!march_fits(g)) return cudaSuccess;
 #define SET(NN, JJ)                                                                       \
   {                                                                                       \
-    const cudaError_t e = allow_max_dyn_smem(march::k_fine_analysis_m<NN, JJ>);           \
+    cudaError_t e = allow_max_dyn_smem(march::k_fine_analysis_m<NN, JJ, true>);           \
+    if (e == cudaSuccess) e = allow_max_dyn_smem(march::k_fine_analysis_m<NN, JJ, false>); \
     return e != cudaSuccess ? e : allow_max_dyn_smem(march::k_fine_adjoint_m<NN, JJ>);    \
   }
   MARCH_CASES(SET)
