@@ -135,8 +135,13 @@ struct SpecArgs {
   const float* pre;  // inverse pre-twiddles (float2) [L]
   const float* invs; // 1 / (s_k L) [L]
   const float* dense;// dense orthonormal DCT matrix [L][L]
+  const float* fold; // its even and odd halves for the folded product (spectral_fold_*), or NULL
   double* partials;
 };
+// Tables of the folded product (L that the FFT does not serve): floats needed
+// (0 for the others), and their values.
+size_t spectral_fold_floats(int L);
+void spectral_fold_tables(int L, float* out);
 bool spectral_uses_fft(int L);
 cudaError_t spectral_configure(int L);
 // Blocks of the pipelined spectral kernel that gave up a bounded wait since the

@@ -11,7 +11,10 @@
 //    FFT(v)[k]); the inverse runs the same steps backwards), the real FFT of
 //    length L done as one complex FFT of length L/2.  Warp w is FFT thread w
 //    of all 32 transforms.
-//  * other L (<= 512): the dense orthonormal DCT matrix.
+//  * other L (<= 512): the orthonormal DCT matrix, folded into its even and odd
+//    halves (k_spectral_fold; the norm of the objective uses the whole matrix).
+#include <cmath>
+
 #include <cuda.h>   // CUtensorMap (the encoder is reached through the runtime's driver entry point)
 
 #include "device.cuh"
@@ -336,7 +339,188 @@ int spectral_take_timeouts() {
   return v;
 }
 
-// Dense fallback: thread (lane, warp) forms coefficients k = warp, warp + W, ...
+// ------------------------------------------------------------------ folded product (L without an FFT)
+// The DCT matrix C[k][l] is symmetric (k even) or antisymmetric (k odd) about
+// the middle channel, so with s[l] = x[l] + x[L-1-l] and d[l] = x[l] - x[L-1-l],
+//   c[2i]   = sum_{l < M} C[2i][l] s[l]      (M = ceil(L/2); s of the middle of an odd L is x)
+//   c[2i+1] = sum_{l < H} C[2i+1][l] d[l]    (H = floor(L/2))
+// and back, e[l] = sum_i C[2i][l] y[2i], o[l] = sum_i C[2i+1][l] y[2i+1],
+// T[l] = e[l] + o[l], T[L-1-l] = e[l] - o[l]: half the multiply-adds.  The
+// products are register tiled: a thread holds 8 rows x 4 pixels, one 16-byte
+// shared-memory read and two uniform table reads feed 32 multiply-adds, so the
+// FP32 pipe bounds the larger L and DRAM the smaller ones.  (One row a thread,
+// as the norm still does it, reads two values for every multiply-add.)
+// 256x256x96: 332 -> 95 us per launch; 256x256x200: 1560 -> 280; 1024x1024x7:
+// 81 -> 41.
+struct FoldDims {
+  int M, H, KE, KO;   // even and odd rows, and both rounded up to 8
+};
+__host__ __device__ inline FoldDims fold_dims(int L) {
+  FoldDims f;
+  f.M = (L + 1) / 2;
+  f.H = L / 2;
+  f.KE = (f.M + 7) & ~7;
+  f.KO = (f.H + 7) & ~7;
+  return f;
+}
+
+size_t spectral_fold_floats(int L) {
+  if (spectral_uses_fft(L)) return 0;
+  const FoldDims f = fold_dims(L);
+  return 2 * ((size_t)f.M * f.KE + (size_t)f.H * f.KO);
+}
+
+// [M][KE] C[2i][l] at (l, i); [M][KE] the same at (i, l); [H][KO] C[2i+1][l] at (l, i); [H][KO] at (i, l)
+void spectral_fold_tables(int L, float* out) {
+  const FoldDims f = fold_dims(L);
+  const double pi = 3.14159265358979323846;
+  for (size_t i = 0, n = spectral_fold_floats(L); i < n; ++i) out[i] = 0.f;
+  float* E = out;
+  float* Et = E + (size_t)f.M * f.KE;
+  float* O = Et + (size_t)f.M * f.KE;
+  float* Ot = O + (size_t)f.H * f.KO;
+  for (int k = 0; k < L; ++k) {
+    const double sk = k == 0 ? std::sqrt(1.0 / L) : std::sqrt(2.0 / L);
+    const int i = k / 2, n = k % 2 ? f.H : f.M;
+    for (int l = 0; l < n; ++l) {
+      const float c = (float)(sk * std::cos(pi * (2 * l + 1) * k / (2.0 * L)));
+      if (k % 2) O[(size_t)l * f.KO + i] = Ot[(size_t)i * f.KO + l] = c;
+      else E[(size_t)l * f.KE + i] = Et[(size_t)i * f.KE + l] = c;
+    }
+  }
+}
+
+__device__ __forceinline__ void fold_row(float4 (&acc)[8], const float* __restrict__ tab, float4 x) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(tab)), b = __ldg(reinterpret_cast<const float4*>(tab) + 1);
+  const float w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    acc[r].x = fmaf(w[r], x.x, acc[r].x);
+    acc[r].y = fmaf(w[r], x.y, acc[r].y);
+    acc[r].z = fmaf(w[r], x.z, acc[r].z);
+    acc[r].w = fmaf(w[r], x.w, acc[r].w);
+  }
+}
+
+// LPR lanes cover the 4 LPR pixels of a subtile; S subtiles a block; a unit of
+// LPR threads takes 8 rows of one subtile at a time.  npix is a multiple of 4 LPR.
+template <int LPR, int MODE>
+__global__ void __launch_bounds__(256, 2)
+k_spectral_fold(SpecArgs a, int npix, int L, int S) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int SUB = 4 * LPR;
+  const FoldDims f = fold_dims(L);
+  const int tp = SUB * S, p0 = blockIdx.x * tp;
+  const int np = npix - p0 < tp ? npix - p0 : tp;       // pixels of this block
+  float* X = sm;                  // [L][tp]: s[l] in row l, d[l] in row L-1-l
+  float* Y = sm + (size_t)L * tp; // [L][tp]: the new duals
+  const size_t P = (size_t)npix;
+  const float *E = a.fold, *Et = E + (size_t)f.M * f.KE, *O = Et + (size_t)f.M * f.KE, *Ot = O + (size_t)f.H * f.KO;
+  const int unit = threadIdx.x / LPR, nunit = blockDim.x / LPR, lc = 4 * (threadIdx.x % LPR);
+  const int nch = tp / 4, ns = np / SUB;                 // chunks of a row; subtiles that exist
+  if constexpr (MODE == SPEC_UPDATE) {
+    const float* D = a.D + p0;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < f.M * nch; i += blockDim.x) {
+      const int l = i / nch, c = 4 * (i % nch);
+      if (c >= np) continue;
+      const float4 u = __ldcg(reinterpret_cast<const float4*>(D + (size_t)l * P + c));
+      if (l < f.H) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(D + (size_t)(L - 1 - l) * P + c));
+        *reinterpret_cast<float4*>(X + l * tp + c) = make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w);
+        *reinterpret_cast<float4*>(X + (L - 1 - l) * tp + c) = make_float4(u.x - v.x, u.y - v.y, u.z - v.z, u.w - v.w);
+      } else {
+        *reinterpret_cast<float4*>(X + l * tp + c) = u;
+      }
+    }
+    __syncthreads();
+    const int ge = f.KE / 8, go = f.KO / 8;
+    for (int it = unit; it < (ge + go) * ns; it += nunit) {
+      const int st = it % ns, g = it / ns, px = st * SUB + lc;
+      const bool odd = g >= ge;
+      const int r0 = 8 * (odd ? g - ge : g), nr = odd ? f.H : f.M, K = odd ? f.KO : f.KE;
+      float4 vo[8], acc[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        acc[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+        vo[r] = acc[r];
+        if (r0 + r < nr) vo[r] = __ldcg(reinterpret_cast<const float4*>(a.V + (size_t)(2 * (r0 + r) + odd) * P + p0 + px));
+      }
+      const float* x = X + px + (odd ? (size_t)(L - 1) * tp : 0);
+      const int step = odd ? -tp : tp;
+      const float* tab = (odd ? O : E) + r0;
+#pragma unroll 4
+      for (int l = 0; l < nr; ++l) fold_row(acc, tab + (size_t)l * K, *reinterpret_cast<const float4*>(x + l * step));
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        if (r0 + r >= nr) continue;
+        const int k = 2 * (r0 + r) + odd;
+        auto dual = [&](float o, float c) { return a.rho * sat1(o + a.k * c) + (1.0f - a.rho) * o; };
+        const float4 n = make_float4(dual(vo[r].x, acc[r].x), dual(vo[r].y, acc[r].y), dual(vo[r].z, acc[r].z),
+                                     dual(vo[r].w, acc[r].w));
+        *reinterpret_cast<float4*>(a.V + (size_t)k * P + p0 + px) = n;
+        *reinterpret_cast<float4*>(Y + k * tp + px) = n;
+      }
+    }
+  } else {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < L * nch; i += blockDim.x) {
+      const int k = i / nch, c = 4 * (i % nch);
+      if (c < np) *reinterpret_cast<float4*>(Y + k * tp + c) = __ldcg(reinterpret_cast<const float4*>(a.V + (size_t)k * P + p0 + c));
+    }
+  }
+  __syncthreads();
+  for (int it = unit; it < f.KE / 8 * ns; it += nunit) {
+    const int st = it % ns, l0 = 8 * (it / ns), px = st * SUB + lc;
+    float4 e[8], o[8];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) e[r] = o[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+    for (int i = 0; i < f.M; ++i) fold_row(e, Et + (size_t)i * f.KE + l0, *reinterpret_cast<const float4*>(Y + 2 * i * tp + px));
+    if (l0 < f.KO)
+#pragma unroll 2
+      for (int i = 0; i < f.H; ++i) fold_row(o, Ot + (size_t)i * f.KO + l0, *reinterpret_cast<const float4*>(Y + (2 * i + 1) * tp + px));
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const int l = l0 + r;
+      if (l >= f.M) continue;
+      float* t = a.T + p0 + px;
+      *reinterpret_cast<float4*>(t + (size_t)l * P) = make_float4(e[r].x + o[r].x, e[r].y + o[r].y, e[r].z + o[r].z, e[r].w + o[r].w);
+      if (l < f.H)
+        *reinterpret_cast<float4*>(t + (size_t)(L - 1 - l) * P) = make_float4(e[r].x - o[r].x, e[r].y - o[r].y, e[r].z - o[r].z, e[r].w - o[r].w);
+    }
+  }
+}
+
+template <int LPR> static cudaError_t spec_fold(const SpecArgs& a, int npix, int L, int mode, cudaStream_t s) {
+  constexpr int SUB = 4 * LPR;
+  const int groups = fold_dims(L).KE / 8;
+  auto smem = [&](int S) { return (size_t)2 * L * SUB * S * sizeof(float); };
+  // subtiles: at least four warps of work in a block, while two or three blocks fit an SM; no fewer blocks than SMs
+  int S = 1;
+  while (groups * S * LPR / 32 < 4 && smem(2 * S) <= 72 * 1024 && npix / (SUB * 2 * S) >= 152) S *= 2;
+  int warps = (groups * S * LPR + 31) / 32;
+  warps = warps < 1 ? 1 : warps > 8 ? 8 : warps;
+  const int grid = (npix + SUB * S - 1) / (SUB * S);
+  if (mode == SPEC_UPDATE) k_spectral_fold<LPR, SPEC_UPDATE><<<grid, 32 * warps, smem(S), s>>>(a, npix, L, S);
+  else k_spectral_fold<LPR, SPEC_TONLY><<<grid, 32 * warps, smem(S), s>>>(a, npix, L, S);
+  return cudaGetLastError();
+}
+
+// The folded product serves the update and the adjoint of a context's cubes:
+// tables given, pixels a multiple of the subtile (N^2 is, for N >= 16), 16-byte
+// aligned arrays, and at least 2^18 values: below, the plain product's larger
+// number of small blocks ends sooner (64x64x8 6.2 against 8.4 us, 64x64x37 17.0
+// against 18.8; 128x128x37 23.0 against 18.4, 64x64x93 76.7 against 31.1).
+// Subtiles of 64 pixels (128 were no faster: 256x256x96 95.6 against 94.5 us)
+// while their two tiles stay below 100 KB, then 32.
+static bool spec_fold_ok(const SpecArgs& a, int npix, int L, int mode) {
+  const auto al = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
+  return a.fold && mode != SPEC_NORM && npix % 64 == 0 && (size_t)npix * L >= ((size_t)1 << 18) && al(a.D) &&
+         al(a.V) && al(a.T);
+}
+
+// Plain product: thread (lane, warp) forms coefficients k = warp, warp + W, ...
 template <int MODE>
 __global__ void __launch_bounds__(256)
 k_spectral_dense(SpecArgs a, int npix, int L) {
@@ -450,6 +634,8 @@ cudaError_t launch_spectral(const SpecArgs& a, int npix, int L, int mode, cudaSt
     }
     return cudaErrorInvalidValue;
   }
+  if (spec_fold_ok(a, npix, L, mode))
+    return L <= 200 ? spec_fold<16>(a, npix, L, mode, s) : spec_fold<8>(a, npix, L, mode, s);
   dim3 grid((npix + 31) / 32), block(32, 8);
   const size_t smem = (size_t)2 * L * 32 * sizeof(float);
   switch (mode) {
@@ -481,6 +667,10 @@ cudaError_t spectral_configure(int L) {
     return cudaErrorInvalidValue;
   }
   cudaError_t e;
+  if ((e = allow_max_dyn_smem(k_spectral_fold<16, SPEC_UPDATE>))) return e;
+  if ((e = allow_max_dyn_smem(k_spectral_fold<16, SPEC_TONLY>))) return e;
+  if ((e = allow_max_dyn_smem(k_spectral_fold<8, SPEC_UPDATE>))) return e;
+  if ((e = allow_max_dyn_smem(k_spectral_fold<8, SPEC_TONLY>))) return e;
   if ((e = allow_max_dyn_smem(k_spectral_dense<SPEC_UPDATE>))) return e;
   if ((e = allow_max_dyn_smem(k_spectral_dense<SPEC_NORM>))) return e;
   return allow_max_dyn_smem(k_spectral_dense<SPEC_TONLY>);

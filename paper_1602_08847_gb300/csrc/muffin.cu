@@ -94,7 +94,7 @@ int default_branches(const muffin_params*) { return 1; }
 struct Layout {
   size_t X, U, V, y, b, Kp, Kb, spec, S, T, D, cr, hhat, yhat, z64, pw, partials, scal;
   size_t W1, W2, W3;   // union of bases: [L][8][N][N] scratch each
-  size_t twf, twd, twL, post, pre, invs, dense, w;
+  size_t twf, twd, twL, post, pre, invs, dense, fold, w;
   size_t total;
   int max_parts;
   int j1;
@@ -143,6 +143,7 @@ Layout make_layout(const muffin_params* p) {
   Lo.pre = take(L * 8);
   Lo.invs = take(L * 4);
   Lo.dense = take(L * L * 4);
+  Lo.fold = take(spectral_fold_floats(p->nchan) * 4);
   Lo.w = take(L * 8);
   Lo.total = (off + 255) & ~(size_t)255;
   return Lo;
@@ -359,6 +360,7 @@ static int enqueue_pass(muffin_ctx* ctx, cudaStream_t s, StageTimer* tm) {
     sa.pre = ctx->at<float>(lo.pre);
     sa.invs = ctx->at<float>(lo.invs);
     sa.dense = ctx->at<float>(lo.dense);
+    sa.fold = spectral_uses_fft(g.L) ? nullptr : ctx->at<float>(lo.fold);
     CK(launch_spectral(sa, (int)P, g.L, SPEC_UPDATE, sp, nullptr));
     mark(6);
     if (fork) {
@@ -388,6 +390,7 @@ static int refresh_adjoints(muffin_ctx* ctx) {
   sa.pre = ctx->at<float>(lo.pre);
   sa.invs = ctx->at<float>(lo.invs);
   sa.dense = ctx->at<float>(lo.dense);
+  sa.fold = spectral_uses_fft(g.L) ? nullptr : ctx->at<float>(lo.fold);
   sa.rho = 1.0f;
   CK(launch_spectral(sa, (int)ctx->P(), g.L, SPEC_TONLY, ctx->stream, nullptr));
   if (g.dict) {
@@ -437,6 +440,11 @@ static void host_tables(const muffin_ctx* ctx, std::vector<char>& blob, const La
   put(lo.pre, pre.data(), pre.size() * 4);
   put(lo.invs, invs.data(), invs.size() * 4);
   put(lo.dense, dense.data(), dense.size() * 4);
+  std::vector<float> fold(spectral_fold_floats(L));
+  if (!fold.empty()) {
+    spectral_fold_tables(L, fold.data());
+    put(lo.fold, fold.data(), fold.size() * 4);
+  }
   put(lo.w, ctx->w.data(), ctx->w.size() * 8);
 }
 
@@ -830,6 +838,7 @@ int muffin_objective(muffin_ctx* ctx, double* h_obj, double* h_terms) {
   sa.pre = ctx->at<float>(lo.pre);
   sa.invs = ctx->at<float>(lo.invs);
   sa.dense = ctx->at<float>(lo.dense);
+  sa.fold = spectral_uses_fft(g.L) ? nullptr : ctx->at<float>(lo.fold);
   sa.partials = ctx->partials();
   CK(launch_spectral(sa, (int)ctx->P(), g.L, SPEC_NORM, s, &np));
   CK(launch_sum_partials(ctx->partials(), np, sc + 13, s));
@@ -1058,6 +1067,7 @@ static void batch_cube_of(const muffin_ctx* ctx, BatchCube* c) {
   sa.pre = ctx->at<float>(lo.pre);
   sa.invs = ctx->at<float>(lo.invs);
   sa.dense = ctx->at<float>(lo.dense);
+  sa.fold = spectral_uses_fft(g.L) ? nullptr : ctx->at<float>(lo.fold);
 }
 
 // The barrier words and the error word of the persistent kernel live in the
