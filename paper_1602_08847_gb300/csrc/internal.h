@@ -117,6 +117,8 @@ struct DwtArgs {
 cudaError_t dwt_configure();
 // mode MODE_UPDATE: U <- rho sat(U + k W_s src) + (1 - rho) U; MODE_LINEAR: U = W_s src.
 cudaError_t launch_dwt_analysis(const Geom& g, const DwtArgs& a, int mode, cudaStream_t s);
+// Kernels of one analysis and one adjoint together.
+int dwt_kernels(const Geom& g);
 // S = W_s^T U.
 cudaError_t launch_dwt_adjoint(const Geom& g, const DwtArgs& a, cudaStream_t s);
 // sum |x| over n floats -> one partial per block (at most 1024).

@@ -12,13 +12,15 @@
 //   g[t] = (-1)^t h[2p-1-t];
 // its adjoint (= inverse, the bank is orthonormal):
 //   x[i] = sum_{t = i mod 2} h[t] lo[k] + g[t] hi[k],  k = ((i - t) mod M) / 2.
-// Every launch covers all channels and all eight bases (gridDim.z = 8 L).
-// The analysis runs one kernel per level, its row and column passes fused
-// through shared memory (a block owns a slab of columns for all rows).  The
-// adjoint runs a column and a row kernel per level, each thread computing a
-// run of outputs (kColRun per thread, kRowsPerBlock rows per block) so that
-// blocks live long enough to amortise their scheduling; the filters have at
-// most 16 taps and those kernels read straight from global memory through L1.
+// Every launch covers all channels and all eight bases.  One kernel per level
+// and direction: a block owns a group of rows over the full width, filters
+// them along one axis into shared memory and from there along the other, each
+// thread a run of outputs with its inputs in registers, so that a value read
+// feeds several multiply-adds (compile-time filter length, taps as constant
+// operands).  The finest level of the adjoint runs the eight bases one after
+// another in a block and sums them in registers, so the per-basis images are
+// never stored.  Levels below 32 x 32 take small kernels that read straight
+// from global memory.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -102,33 +104,12 @@ bool daubechies_lowpass(int p, double* h) {
   return true;
 }
 
-cudaError_t dwt_configure() {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  static bool done[64] = {};
-  if (dev < 64 && done[dev]) return cudaSuccess;
-  float hf[kDbBases][kMaxTaps] = {}, gf[kDbBases][kMaxTaps] = {};
-  for (int b = 0; b < kDbBases; ++b) {
-    double h[kMaxTaps];
-    const int p = b + 1, taps = 2 * p;
-    daubechies_lowpass(p, h);
-    for (int t = 0; t < taps; ++t) {
-      hf[b][t] = (float)h[t];
-      gf[b][t] = (float)((t & 1 ? -1.0 : 1.0) * h[taps - 1 - t]);
-    }
-  }
-  if ((e = cudaMemcpyToSymbol(c_dbh, hf, sizeof(hf))) != cudaSuccess) return e;
-  if ((e = cudaMemcpyToSymbol(c_dbg, gf, sizeof(gf))) != cudaSuccess) return e;
-  if (dev < 64) done[dev] = true;
-  return cudaSuccess;
-}
-
 // ------------------------------------------------------------------ kernels
 
 constexpr float kUnionScale = 0.35355339059327373f;   // 1/sqrt(8)
 constexpr int kRowsPerBlock = 8;
 constexpr int kColRun = 4;
+constexpr int kMinTile = 32;      // smallest level of the row-group kernels
 
 // The kernels below run one body per basis, instantiated for its filter length
 // (TAPS = 2p, compile time) so that every tap loop unrolls and its loads issue
@@ -144,6 +125,204 @@ constexpr int kColRun = 4;
     case 6: CALL(14); break;     \
     default: CALL(16); break;    \
   }
+
+// ------------------------------------------------------------------ row-group kernels, levels of at least 32 x 32
+//
+// 256 x 256 x 64, four levels, us per pass: analysis 258 -> 157, adjoint 399 ->
+// 117, bitwise the same (before: a thread per output, one load for every one or
+// two multiply-adds, and for the adjoint columns and rows in separate kernels
+// with the images between them in global memory).  The analysis is bound by the
+// L1 reads of its row filter and the read-modify-write of U (40 us of DRAM at
+// copy speed), the adjoint by the FP32 pipe at 16 warps per SM.
+
+// Analysis of level M: rows q0 .. q0 + Q - 1 of the low and of the high half,
+// from the input rows 2 q0 .. 2 q0 + 2Q + TAPS - 3.  Shared: those rows after
+// the row filter, [row][M] (low columns, then high ones).
+template <int MODE, int TAPS, int Q>
+__device__ __forceinline__ void dwt_rows_body(const float* __restrict__ src, float* __restrict__ ll,
+                                              float* __restrict__ U, int n, int M, int last, float kk, float rho,
+                                              float* __restrict__ sY) {
+  constexpr int b = TAPS / 2 - 1, ROWS = 2 * Q + TAPS - 2, NV = (8 + TAPS - 2 + 3) / 4;
+  const int H = M >> 1, m = M - 1, q0 = blockIdx.x * Q;
+  // rows: an item is four low and four high outputs of a row, from 8 + TAPS - 2 inputs
+  const int runs = M >> 3;
+  for (int it = threadIdx.x; it < ROWS * runs; it += blockDim.x) {
+    const int r = it / runs, k0 = 4 * (it - r * runs);
+    const float* row = src + (size_t)((2 * q0 + r) & m) * n;
+    float x[4 * NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const float4 t = __ldg(reinterpret_cast<const float4*>(row + ((2 * k0 + 4 * v) & m)));
+      x[4 * v] = t.x; x[4 * v + 1] = t.y; x[4 * v + 2] = t.z; x[4 * v + 3] = t.w;
+    }
+    float lo[4] = {}, hi[4] = {};
+#pragma unroll
+    for (int t = 0; t < TAPS; ++t)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        lo[e] = fmaf(c_dbh[b][t], x[2 * e + t], lo[e]);
+        hi[e] = fmaf(c_dbg[b][t], x[2 * e + t], hi[e]);
+      }
+    *reinterpret_cast<float4*>(sY + r * M + k0) = make_float4(lo[0], lo[1], lo[2], lo[3]);
+    *reinterpret_cast<float4*>(sY + r * M + H + k0) = make_float4(hi[0], hi[1], hi[2], hi[3]);
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < M; c += blockDim.x) {
+    const bool keep = c < H && !last;            // the low-low quadrant feeds the next level
+    float* ul = U + (size_t)q0 * n + c;
+    float* uh = ul + (size_t)H * n;
+    float ol[Q], oh[Q];                           // old duals, loaded under the column filter
+    if (MODE == MODE_UPDATE) {
+#pragma unroll
+      for (int q = 0; q < Q; ++q) {
+        ol[q] = keep ? 0.f : ul[(size_t)q * n];
+        oh[q] = uh[(size_t)q * n];
+      }
+    }
+    float x[ROWS];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) x[r] = sY[r * M + c];
+    auto dual = [&](float o, float w) {
+      w *= kUnionScale;
+      return MODE == MODE_UPDATE ? rho * sat1(o + kk * w) + (1.0f - rho) * o : w;
+    };
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      float lo = 0.f, hi = 0.f;
+#pragma unroll
+      for (int t = 0; t < TAPS; ++t) {
+        lo = fmaf(c_dbh[b][t], x[2 * q + t], lo);
+        hi = fmaf(c_dbg[b][t], x[2 * q + t], hi);
+      }
+      if (keep) ll[(size_t)(q0 + q) * n + c] = lo;
+      else ul[(size_t)q * n] = dual(ol[q], lo);
+      uh[(size_t)q * n] = dual(oh[q], hi);
+    }
+  }
+}
+
+// grid (M / 2 / Q, 1, 8 L); shared (2Q + 14) M floats
+template <int MODE, int Q>
+__global__ void __launch_bounds__(512)
+k_dwt_rows(const float* __restrict__ src0, const float* __restrict__ llin, float* __restrict__ ll,
+           float* __restrict__ U, int n, int M, int level0, int last, float kk, float rho) {
+  extern __shared__ __align__(16) float sY[];
+  const size_t P = (size_t)n * n;
+  const int z = blockIdx.z;
+  const float* src = level0 ? src0 + (size_t)(z >> 3) * P : llin + (size_t)z * P;
+#define CALL(T) dwt_rows_body<MODE, T, Q>(src, ll + (size_t)z * P, U + (size_t)z * P, n, M, last, kk, rho, sY)
+  MUFFIN_DB_DISPATCH(CALL)
+#undef CALL
+}
+
+// Shared slot of column x: four spare floats after every 32, so that the
+// 16-byte reads of lanes 32 bytes apart fall into different banks.
+__device__ __forceinline__ int syn_slot(int x) { return x + ((x >> 5) << 2); }
+__host__ __device__ constexpr int syn_pitch(int M) { return M + M / 8; }
+
+// Adjoint of one basis and level M for output rows 2 q0 .. 2 q0 + R - 1: adds
+// this thread's 16 outputs (row, 16 columns from 16 run) to acc.  lo / hi of
+// column c: rows of the low-low image (c < H, unless this is the coarsest
+// level) or of U, and rows H .. of U.  Shared: [R][syn_pitch(M)].
+template <int TAPS, int R>
+__device__ __forceinline__ void idwt_group(const float* __restrict__ U, const float* __restrict__ llin, int n, int M,
+                                           int q0, int coarsest, float* __restrict__ sV, int row, int run,
+                                           float (&acc)[16]) {
+  constexpr int b = TAPS / 2 - 1, p = TAPS / 2, NQ = R / 2, NW = (p - 1 + 3) / 4;   // NW chunks before the run
+  const int H = M >> 1, hm = H - 1, pitch = syn_pitch(M);
+  for (int c = threadIdx.x; c < M; c += blockDim.x) {
+    const float* lo = (c < H && !coarsest ? llin : U) + c;
+    const float* hi = U + (size_t)H * n + c;
+    float a[NQ + p - 1], d[NQ + p - 1];
+#pragma unroll
+    for (int i = 0; i < NQ + p - 1; ++i) {
+      const size_t k = (size_t)((q0 - (p - 1) + i) & hm) * n;
+      a[i] = __ldg(lo + k);
+      d[i] = __ldg(hi + k);
+    }
+#pragma unroll
+    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+      for (int par = 0; par < 2; ++par) {
+        float v = 0.f;
+#pragma unroll
+        for (int s = 0; s < p; ++s) {
+          v = fmaf(c_dbh[b][par + 2 * s], a[q + p - 1 - s], v);
+          v = fmaf(c_dbg[b][par + 2 * s], d[q + p - 1 - s], v);
+        }
+        sV[(2 * q + par) * pitch + syn_slot(c)] = v;
+      }
+  }
+  __syncthreads();
+  const float* vr = sV + row * pitch;
+  const int u0 = 8 * run;
+  float a[4 * NW + 8], d[4 * NW + 8];
+#pragma unroll
+  for (int i = 0; i < NW + 2; ++i) {
+    const int u = (u0 - 4 * NW + 4 * i) & hm;
+    const float4 x = *reinterpret_cast<const float4*>(vr + syn_slot(u));
+    const float4 y = *reinterpret_cast<const float4*>(vr + syn_slot(H + u));
+    a[4 * i] = x.x; a[4 * i + 1] = x.y; a[4 * i + 2] = x.z; a[4 * i + 3] = x.w;
+    d[4 * i] = y.x; d[4 * i + 1] = y.y; d[4 * i + 2] = y.z; d[4 * i + 3] = y.w;
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e)
+#pragma unroll
+    for (int par = 0; par < 2; ++par) {
+      float v = 0.f;
+#pragma unroll
+      for (int s = 0; s < p; ++s) {
+        v = fmaf(c_dbh[b][par + 2 * s], a[4 * NW + e - s], v);
+        v = fmaf(c_dbg[b][par + 2 * s], d[4 * NW + e - s], v);
+      }
+      acc[2 * e + par] += v;
+    }
+  __syncthreads();       // the next basis overwrites sV
+}
+
+__device__ __forceinline__ void put16(float* __restrict__ o, const float (&v)[16], float k) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    reinterpret_cast<float4*>(o)[i] = make_float4(k * v[4 * i], k * v[4 * i + 1], k * v[4 * i + 2], k * v[4 * i + 3]);
+}
+
+// One level and basis: grid (M / R, 1, 8 L), M R / 16 threads.
+template <int R>
+__global__ void __launch_bounds__(512)
+k_idwt_group(const float* __restrict__ U, const float* __restrict__ llin, float* __restrict__ out, int n, int M,
+             int coarsest) {
+  extern __shared__ __align__(16) float sV[];
+  const size_t z = blockIdx.z, P = (size_t)n * n;
+  const int row = threadIdx.x / (M >> 4), run = threadIdx.x % (M >> 4);
+  float acc[16] = {};
+#define CALL(T) idwt_group<T, R>(U + z * P, llin + z * P, n, M, blockIdx.x * (R / 2), coarsest, sV, row, run, acc)
+  MUFFIN_DB_DISPATCH(CALL)
+#undef CALL
+  put16(out + z * P + (size_t)(blockIdx.x * R + row) * n + 16 * run, acc, 1.0f);
+}
+
+// Finest level, all eight bases: S = (1/sqrt 8) sum_b.  grid (N / R, 1, L).
+template <int R>
+__global__ void __launch_bounds__(512)
+k_idwt_group_sum(const float* __restrict__ U, const float* __restrict__ llin, float* __restrict__ S, int n,
+                 int coarsest) {
+  extern __shared__ __align__(16) float sV[];
+  const size_t l = blockIdx.z, P = (size_t)n * n;
+  const int row = threadIdx.x / (n >> 4), run = threadIdx.x % (n >> 4), q0 = blockIdx.x * (R / 2);
+  const float *u = U + l * kDbBases * P, *w = llin + l * kDbBases * P;
+  float acc[16] = {};
+  idwt_group<2, R>(u, w, n, n, q0, coarsest, sV, row, run, acc);
+  idwt_group<4, R>(u + P, w + P, n, n, q0, coarsest, sV, row, run, acc);
+  idwt_group<6, R>(u + 2 * P, w + 2 * P, n, n, q0, coarsest, sV, row, run, acc);
+  idwt_group<8, R>(u + 3 * P, w + 3 * P, n, n, q0, coarsest, sV, row, run, acc);
+  idwt_group<10, R>(u + 4 * P, w + 4 * P, n, n, q0, coarsest, sV, row, run, acc);
+  idwt_group<12, R>(u + 5 * P, w + 5 * P, n, n, q0, coarsest, sV, row, run, acc);
+  idwt_group<14, R>(u + 6 * P, w + 6 * P, n, n, q0, coarsest, sV, row, run, acc);
+  idwt_group<16, R>(u + 7 * P, w + 7 * P, n, n, q0, coarsest, sV, row, run, acc);
+  put16(S + l * P + (size_t)(blockIdx.x * R + row) * n + 16 * run, acc, kUnionScale);
+}
+
+// ------------------------------------------------------------------ small levels
 
 // Analysis of one whole level, rows and columns fused through shared memory.
 // A block owns a slab of SC consecutive columns k0 .. k0 + SC - 1 of the
@@ -375,6 +554,33 @@ __global__ void k_abs_sum(const float* __restrict__ x, size_t n, double* __restr
   if (threadIdx.x == 0) partials[blockIdx.x] = t;
 }
 
+cudaError_t dwt_configure() {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  static bool done[64] = {};
+  if (dev < 64 && done[dev]) return cudaSuccess;
+  float hf[kDbBases][kMaxTaps] = {}, gf[kDbBases][kMaxTaps] = {};
+  for (int b = 0; b < kDbBases; ++b) {
+    double h[kMaxTaps];
+    const int p = b + 1, taps = 2 * p;
+    daubechies_lowpass(p, h);
+    for (int t = 0; t < taps; ++t) {
+      hf[b][t] = (float)h[t];
+      gf[b][t] = (float)((t & 1 ? -1.0 : 1.0) * h[taps - 1 - t]);
+    }
+  }
+  if ((e = cudaMemcpyToSymbol(c_dbh, hf, sizeof(hf))) != cudaSuccess) return e;
+  if ((e = cudaMemcpyToSymbol(c_dbg, gf, sizeof(gf))) != cudaSuccess) return e;
+  if ((e = allow_max_dyn_smem(k_dwt_rows<MODE_UPDATE, 8>)) != cudaSuccess) return e;
+  if ((e = allow_max_dyn_smem(k_dwt_rows<MODE_LINEAR, 8>)) != cudaSuccess) return e;
+  if ((e = allow_max_dyn_smem(k_idwt_group<16>)) != cudaSuccess) return e;
+  if ((e = allow_max_dyn_smem(k_idwt_group_sum<16>)) != cudaSuccess) return e;
+  if ((e = allow_max_dyn_smem(k_idwt_group_sum<8>)) != cudaSuccess) return e;
+  if (dev < 64) done[dev] = true;
+  return cudaSuccess;
+}
+
 // ------------------------------------------------------------------ launchers
 
 // Columns per slab of the fused analysis: at most 32, at most 8192 / M (32 KB
@@ -385,34 +591,62 @@ static int dwt_slab(int M) {
   return sc;
 }
 
+template <int MODE>
+static void dwt_level(const Geom& g, const DwtArgs& a, int j, cudaStream_t s) {
+  const int n = g.n, Z = kDbBases * g.L, M = n >> j, last = j == g.J - 1;
+  // level j reads the low-low plane level j - 1 wrote and writes its own to the other scratch plane
+  const float* llin = (j & 1) ? a.W1 : a.W2;
+  float* ll = (j & 1) ? a.W2 : a.W1;
+  const float kk = MODE == MODE_UPDATE ? a.k : 1.f, rho = MODE == MODE_UPDATE ? a.rho : 1.f;
+  if (M >= kMinTile) {
+    // eight output rows of each half a block (their 16 + TAPS - 2 input rows overlap the next block's by TAPS - 2)
+    constexpr int Q = 8;
+    k_dwt_rows<MODE, Q><<<dim3(M / 2 / Q, 1, Z), M < 512 ? M : 512, (size_t)(2 * Q + kMaxTaps - 2) * M * sizeof(float), s>>>(
+        a.src, llin, ll, a.U, n, M, j == 0, last, kk, rho);
+  } else {
+    const int sc = dwt_slab(M);
+    k_dwt_level<MODE><<<dim3(M / sc, 1, Z), 256, (size_t)M * sc * sizeof(float), s>>>(a.src, llin, ll, a.U, n, M, sc,
+                                                                                  j == 0, last, kk, rho);
+  }
+}
+
 cudaError_t launch_dwt_analysis(const Geom& g, const DwtArgs& a, int mode, cudaStream_t s) {
-  const int n = g.n, Z = kDbBases * g.L;
   for (int j = 0; j < g.J; ++j) {
-    const int M = n >> j, sc = dwt_slab(M);
-    // level j reads the low-low plane level j - 1 wrote and writes its own to the other scratch plane
-    const float* llin = (j & 1) ? a.W1 : a.W2;
-    float* ll = (j & 1) ? a.W2 : a.W1;
-    const dim3 grid(M / sc, 1, Z);
-    const size_t sm = (size_t)M * sc * sizeof(float);
-    const int last = j == g.J - 1;
-    if (mode == MODE_UPDATE)
-      k_dwt_level<MODE_UPDATE><<<grid, 256, sm, s>>>(a.src, llin, ll, a.U, n, M, sc, j == 0, last, a.k, a.rho);
-    else
-      k_dwt_level<MODE_LINEAR><<<grid, 256, sm, s>>>(a.src, llin, ll, a.U, n, M, sc, j == 0, last, 1.f, 1.f);
+    if (mode == MODE_UPDATE) dwt_level<MODE_UPDATE>(g, a, j, s);
+    else dwt_level<MODE_LINEAR>(g, a, j, s);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_dwt_adjoint(const Geom& g, const DwtArgs& a, cudaStream_t s) {
   const int n = g.n, Z = kDbBases * g.L;
+  const float* in = a.W2;       // low-low images of the level before
   for (int j = g.J - 1; j >= 0; --j) {
-    const int M = n >> j;
+    const int M = n >> j, coarsest = j == g.J - 1;
+    if (M >= kMinTile) {
+      float* out = j == 0 ? a.S : in == a.W1 ? a.W2 : a.W1;
+      // rows per group: 16, as many threads as columns; 8 at 1024 columns (512 threads, two columns each)
+      const size_t sm = (size_t)syn_pitch(M) * sizeof(float);
+      if (j > 0) k_idwt_group<16><<<dim3(M / 16, 1, Z), M, 16 * sm, s>>>(a.U, in, out, n, M, coarsest);
+      else if (M == 1024) k_idwt_group_sum<8><<<dim3(M / 8, 1, g.L), 512, 8 * sm, s>>>(a.U, in, out, n, coarsest);
+      else k_idwt_group_sum<16><<<dim3(M / 16, 1, g.L), M, 16 * sm, s>>>(a.U, in, out, n, coarsest);
+      in = out;
+      continue;
+    }
+    // small levels come first and hand their images on in W2
     k_idwt_cols<<<dim3((M + 31) / 32, (M + 8 * kColRun - 1) / (8 * kColRun), Z), dim3(32, 8), 0, s>>>(
-        a.U, a.W2, a.W1, n, M, j == g.J - 1);
+        a.U, a.W2, a.W1, n, M, coarsest);
     if (j > 0) k_idwt_rows<<<dim3(1, (M + kRowsPerBlock - 1) / kRowsPerBlock, Z), 128, 0, s>>>(a.W1, a.W2, n, M);
     else k_idwt_rows_sum<<<dim3(1, (M + kRowsPerBlock - 1) / kRowsPerBlock, g.L), 256, 0, s>>>(a.W1, a.S, n);
   }
   return cudaGetLastError();
+}
+
+// Kernels that one analysis and one adjoint launch.
+int dwt_kernels(const Geom& g) {
+  int k = g.J;
+  for (int j = 0; j < g.J; ++j) k += (g.n >> j) >= kMinTile ? 1 : 2;
+  return k;
 }
 
 cudaError_t launch_abs_sum(const float* x, size_t n, double* partials, int* nparts, cudaStream_t s) {

@@ -958,7 +958,7 @@ int muffin_kernels_per_iteration(const muffin_ctx* ctx) {
   int per_group = 0;
   for (int k = 0; k < kNumStages; ++k) per_group += (k != 6 && muffin_stage_bytes(ctx, k) > 0) ? 1 : 0;
   int n = ngroups * per_group + (muffin_stage_bytes(ctx, 6) > 0 ? 1 : 0);
-  if (ctx->g.dict && ctx->mu_s != 0.0) n += 3 * ctx->g.J - 2;   // 2J adjoint and J analysis kernels, not 2
+  if (ctx->g.dict && ctx->mu_s != 0.0) n += dwt_kernels(ctx->g) - 2;   // counted as 2 so far
   return n;
 }
 
