@@ -42,14 +42,16 @@ cudaError_t launch_rows_inv_primal(const float* spec, const PrimalArgs& a, int n
                                    cudaStream_t s);
 cudaError_t launch_rows_inv_plain(const float* spec, float* out, int n, int L, const float* twf, cudaStream_t s);
 
-// FP64 full-complex 2-D FFT helpers for setup and the objective.
-// mode_in: 0 complex input z; 1 real float input with ifftshift; 2 real float input.
-cudaError_t launch_c2c_rows64(const void* in, int mode_in, void* z, int n, int L, int dir, const void* twd,
+// FP64 2-D FFT helpers for setup and the objective, on the bins kx = 0 .. N/2
+// of [L][N][N] complex arrays (the others are neither written nor read).
+// mode_in: 1 a PSF, moved by (N/2, N/2); 2 a cube as it is.
+cudaError_t launch_r2c_rows64(const float* in, int mode_in, void* z, int n, int L, const void* twd, cudaStream_t s);
+// out = w_l / N^2 times the inverse row transform, float32
+cudaError_t launch_c2r_rows64(const void* z, const double* w, float* out, int n, int L, const void* twd,
                               cudaStream_t s);
 cudaError_t launch_c2c_cols64(void* z, int n, int L, int dir, const void* twd, cudaStream_t s);
 cudaError_t launch_build_K(const void* hhat, const double* w, float* Kp, float* Kb, int n, int L, cudaStream_t s);
 cudaError_t launch_mul_conj(const void* hhat, void* z, int n, int L, cudaStream_t s);
-cudaError_t launch_real_to_float(const void* z, const double* w, float* out, int n, int L, cudaStream_t s);
 // sum_l w_l / (2 N^2) sum_k |hhat z - yhat|^2 over column tiles -> partials
 cudaError_t launch_cols64_fidelity(void* z, const void* hhat, const void* yhat, const double* w, int n, int L,
                                    const void* twd, double* partials, int* nparts, cudaStream_t s);

@@ -651,17 +651,16 @@ int muffin_set_psf(muffin_ctx* ctx, const float* d_psf) {
   const void* twd = ctx->ws + lo.twd;
   const double* w = ctx->at<double>(lo.w);
   // hhat_l = DFT of the PSF moved to the origin; yhat_l = DFT of y_l (FP64)
-  CK(launch_c2c_rows64(d_psf, 1, hh, n, L, -1, twd, s));
+  CK(launch_r2c_rows64(d_psf, 1, hh, n, L, twd, s));
   CK(launch_c2c_cols64(hh, n, L, -1, twd, s));
-  CK(launch_c2c_rows64(ctx->at<float>(lo.y), 2, yh, n, L, -1, twd, s));
+  CK(launch_r2c_rows64(ctx->at<float>(lo.y), 2, yh, n, L, twd, s));
   CK(launch_c2c_cols64(yh, n, L, -1, twd, s));
   CK(launch_build_K(hh, w, ctx->at<float>(lo.Kp), ctx->at<float>(lo.Kb), n, L, s));
   // b_l = w_l H_l^T y_l = w_l IDFT(conj(hhat) yhat)
   CK(cudaMemcpyAsync(z, yh, V * 16, cudaMemcpyDeviceToDevice, s));
   CK(launch_mul_conj(hh, z, n, L, s));
   CK(launch_c2c_cols64(z, n, L, 1, twd, s));
-  CK(launch_c2c_rows64(z, 0, z, n, L, 1, twd, s));
-  CK(launch_real_to_float(z, w, ctx->at<float>(lo.b), n, L, s));
+  CK(launch_c2r_rows64(z, w, ctx->at<float>(lo.b), n, L, twd, s));
   int np = 0;
   CK(launch_max_abs2(hh, w, n, L, ctx->partials(), &np, s));
   CK(launch_max_partials(ctx->partials(), np, sc + 0, s));
@@ -678,8 +677,10 @@ int muffin_set_psf(muffin_ctx* ctx, const float* d_psf) {
     CK(launch_rows_fwd(pv, spec, n, L, twf, s));
     CK(launch_cols_filter(spec, ctx->at<float>(lo.Kp), ctx->at<float>(lo.Kb), n, L, twf, s));
     CK(launch_rows_inv_plain(spec, pw, n, L, twf, s));
-    CK(launch_dot(pv, pw, V, ctx->partials(), &np, s));
-    CK(launch_sum_partials(ctx->partials(), np, sc + 2, s));
+    if (it == ctx->p.power_iters - 1) {      // the estimate <v, H^T H v> is the last pass's
+      CK(launch_dot(pv, pw, V, ctx->partials(), &np, s));
+      CK(launch_sum_partials(ctx->partials(), np, sc + 2, s));
+    }
     CK(launch_dot(pw, pw, V, ctx->partials(), &np, s));
     CK(launch_sum_partials(ctx->partials(), np, sc + 1, s));
     CK(launch_scale(pw, V, nullptr, sc + 1, s));
@@ -704,14 +705,18 @@ int muffin_set_psf(muffin_ctx* ctx, const float* d_psf) {
     CK(launch_sum_partials(ctx->partials(), np, sc + 4, s));
     CK(launch_scale(x, P, nullptr, sc + 4, s));
     for (int it = 0; it < ctx->p.power_iters; ++it) {
+      da.src = x;
+      da.S = St;
       CK(launch_dwt_analysis(g1, da, MODE_LINEAR, s));
       CK(launch_dwt_adjoint(g1, da, s));
-      CK(launch_dot(x, St, P, ctx->partials(), &np, s));
-      CK(launch_sum_partials(ctx->partials(), np, sc + 3, s));
+      if (it == ctx->p.power_iters - 1) {
+        CK(launch_dot(x, St, P, ctx->partials(), &np, s));
+        CK(launch_sum_partials(ctx->partials(), np, sc + 3, s));
+      }
       CK(launch_dot(St, St, P, ctx->partials(), &np, s));
       CK(launch_sum_partials(ctx->partials(), np, sc + 4, s));
-      CK(cudaMemcpyAsync(x, St, P * 4, cudaMemcpyDeviceToDevice, s));
-      CK(launch_scale(x, P, nullptr, sc + 4, s));
+      CK(launch_scale(St, P, nullptr, sc + 4, s));
+      std::swap(x, St);
     }
   } else if (g.J > 0) {
     Geom g1 = g;
@@ -727,16 +732,20 @@ int muffin_set_psf(muffin_ctx* ctx, const float* d_psf) {
     CK(launch_sum_partials(ctx->partials(), np, sc + 4, s));
     CK(launch_scale(x, P, nullptr, sc + 4, s));
     for (int it = 0; it < ctx->p.power_iters; ++it) {
+      ia.D = x;
+      ia.S = St;
       if (g1.j1 > 0) CK(launch_fine_analysis(g1, ia, MODE_LINEAR, s, nullptr));
       if (g1.J > g1.j1)
         CK(launch_coarse(g1, g1.j1 > 0 ? crt : x, g1.j1 > 0 ? crt : St, Ut, 1.f, 1.f, MODE_LINEAR, nullptr, s, nullptr));
       if (g1.j1 > 0) CK(launch_fine_adjoint(g1, ia, s));
-      CK(launch_dot(x, St, P, ctx->partials(), &np, s));
-      CK(launch_sum_partials(ctx->partials(), np, sc + 3, s));
+      if (it == ctx->p.power_iters - 1) {
+        CK(launch_dot(x, St, P, ctx->partials(), &np, s));
+        CK(launch_sum_partials(ctx->partials(), np, sc + 3, s));
+      }
       CK(launch_dot(St, St, P, ctx->partials(), &np, s));
       CK(launch_sum_partials(ctx->partials(), np, sc + 4, s));
-      CK(cudaMemcpyAsync(x, St, P * 4, cudaMemcpyDeviceToDevice, s));
-      CK(launch_scale(x, P, nullptr, sc + 4, s));
+      CK(launch_scale(St, P, nullptr, sc + 4, s));
+      std::swap(x, St);
     }
   }
   double h[4] = {0, 0, 0, 0};
@@ -807,7 +816,7 @@ int muffin_objective(muffin_ctx* ctx, double* h_obj, double* h_terms) {
   void* z = ctx->ws + lo.z64;
   int np = 0;
   CK(cudaMemsetAsync(sc + 10, 0, 4 * sizeof(double), s));
-  CK(launch_c2c_rows64(ctx->X(), 2, z, g.n, g.L, -1, ctx->ws + lo.twd, s));
+  CK(launch_r2c_rows64(ctx->X(), 2, z, g.n, g.L, ctx->ws + lo.twd, s));
   CK(launch_cols64_fidelity(z, ctx->ws + lo.hhat, ctx->ws + lo.yhat, ctx->at<double>(lo.w), g.n, g.L,
                             ctx->ws + lo.twd, ctx->partials(), &np, s));
   CK(launch_sum_partials(ctx->partials(), np, sc + 10, s));
