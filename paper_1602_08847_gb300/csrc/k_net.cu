@@ -911,15 +911,13 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
 
 // ------------------------------------------------------------------ first and last layers (CUDA cores)
 
-// Thread -> voxel (tz, ty, tx) of the tile.
-__device__ __forceinline__ void thread_voxel(int& tz, int& ty, int& tx) {
-  tx = threadIdx.x & 15;
-  ty = (threadIdx.x >> 4) & 7;
-  tz = threadIdx.x >> 7;
-}
-
-// a1[p][co] = relu(b[co] + sum_tap a0[p + d(tap)] w[tap][co]).
-__global__ void __launch_bounds__(256)
+// a1[p][co] = relu(b[co] + sum_tap a0[p + d(tap)] w[tap][co]).  A thread takes
+// the two channels z of one (row, column) of the tile, so that the 32 weights
+// of a tap, read once, feed 64 multiply-adds (one channel a thread: as many
+// shared-memory reads as groups of four multiply-adds, 0.342 against 0.244 ms
+// at 64x256x256).
+constexpr int kFirstThreads = TY * TX;
+__global__ void __launch_bounds__(kFirstThreads)
 k_first_fwd(const bf16* __restrict__ a0, const float* __restrict__ w, const float* __restrict__ b,
             bf16* __restrict__ a1, Dims d) {
   __shared__ __align__(16) float s_w[NTAP * C];
@@ -927,58 +925,76 @@ k_first_fwd(const bf16* __restrict__ a0, const float* __restrict__ w, const floa
   __shared__ float s_h[HV];
   for (int i = threadIdx.x; i < NTAP * C; i += blockDim.x) s_w[i] = w[i];
   if (threadIdx.x < C) s_b[threadIdx.x] = b[threadIdx.x];
-  int tz, ty, tx;
-  thread_voxel(tz, ty, tx);
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
   for (int tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) {
     int z0, y0, x0;
     tile_origin(tile, d, z0, y0, x0);
     __syncthreads();
     load_scalar_halo(s_h, a0, d, z0, y0, x0);
     __syncthreads();
-    float acc[C];
+    float acc[TZ][C];
 #pragma unroll
-    for (int c = 0; c < C; ++c) acc[c] = s_b[c];
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int z = 0; z < TZ; ++z) acc[z][c] = s_b[c];
 #pragma unroll 1
     for (int t = 0; t < NTAP; ++t) {
       const int kz = t / 9, ky = (t / 3) % 3, kx = t % 3;
-      const float av = s_h[((tz + kz) * HY + ty + ky) * HX + tx + kx];
+      float av[TZ];
+#pragma unroll
+      for (int z = 0; z < TZ; ++z) av[z] = s_h[((z + kz) * HY + ty + ky) * HX + tx + kx];
       const float4* wr = reinterpret_cast<const float4*>(s_w + t * C);
 #pragma unroll
       for (int q = 0; q < C / 4; ++q) {
         const float4 wv = wr[q];
-        acc[4 * q] = fmaf(av, wv.x, acc[4 * q]);
-        acc[4 * q + 1] = fmaf(av, wv.y, acc[4 * q + 1]);
-        acc[4 * q + 2] = fmaf(av, wv.z, acc[4 * q + 2]);
-        acc[4 * q + 3] = fmaf(av, wv.w, acc[4 * q + 3]);
+#pragma unroll
+        for (int z = 0; z < TZ; ++z) {
+          acc[z][4 * q] = fmaf(av[z], wv.x, acc[z][4 * q]);
+          acc[z][4 * q + 1] = fmaf(av[z], wv.y, acc[z][4 * q + 1]);
+          acc[z][4 * q + 2] = fmaf(av[z], wv.z, acc[z][4 * q + 2]);
+          acc[z][4 * q + 3] = fmaf(av[z], wv.w, acc[z][4 * q + 3]);
+        }
       }
     }
-    const int z = z0 + tz, y = y0 + ty, x = x0 + tx;
-    if (inside(d, z, y, x)) {
 #pragma unroll
-      for (int c = 0; c < C; ++c) acc[c] = fmaxf(acc[c], 0.f);
-      uint4* o = reinterpret_cast<uint4*>(a1 + vox(d, z, y, x) * C);
+    for (int z = 0; z < TZ; ++z) {
+      if (!inside(d, z0 + z, y0 + ty, x0 + tx)) continue;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) o[q] = pack8(acc + 8 * q);
+      for (int c = 0; c < C; ++c) acc[z][c] = fmaxf(acc[z][c], 0.f);
+      uint4* o = reinterpret_cast<uint4*>(a1 + vox(d, z0 + z, y0 + ty, x0 + tx) * C);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) o[q] = pack8(acc[z] + 8 * q);
     }
   }
 }
 
 // part[b][tap][co] = sum_p g1[p][co] a0[p + d(tap)]; bpart[b][co] = sum_p g1[p][co].
-// 288 threads: thread (kz, ky, co) keeps the three taps kx = 0..2 of its row
-// offset and walks each tile row along x with a sliding window of three a0
-// values (one a0 and one g1 read per 3 multiply-adds).
-__global__ void __launch_bounds__(288)
+// Lane = co; each of the eight warps takes two tile rows of sixteen voxels and
+// keeps all 27 taps in registers: four voxels' g1 values and, row offset by row
+// offset, eight a0 values (two 16-byte reads, the same for every lane) feed 12
+// multiply-adds.  (A warp per row offset read one a0 and one g1 value for every
+// three: 0.509 against 0.281 ms at 64x256x256.)  The warps' sums are added in a
+// fixed order at the end.
+constexpr int HXP = 20;     // halo row pitch: 18 columns, 16-byte aligned rows
+__global__ void __launch_bounds__(256, 3)
 k_wgrad_first(const bf16* __restrict__ a0, const bf16* __restrict__ g1, float* __restrict__ part,
               float* __restrict__ bpart, Dims d) {
-  __shared__ float s_h[HV];
+  __shared__ __align__(16) float s_h[HZ * HY * HXP];
   __shared__ __align__(16) float s_g[TV * C];
-  const int co = threadIdx.x & 31, kzy = threadIdx.x >> 5, kz = kzy / 3, ky = kzy % 3;
-  float acc0 = 0.f, acc1 = 0.f, acc2 = 0.f, bacc = 0.f;
+  const int co = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float acc[NTAP], bacc = 0.f;
+#pragma unroll
+  for (int t = 0; t < NTAP; ++t) acc[t] = 0.f;
+  for (int i = threadIdx.x; i < HZ * HY * HXP; i += blockDim.x) s_h[i] = 0.f;     // the pad columns stay zero
   for (int tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) {
     int z0, y0, x0;
     tile_origin(tile, d, z0, y0, x0);
     __syncthreads();
-    load_scalar_halo(s_h, a0, d, z0, y0, x0);
+    for (int h = threadIdx.x; h < HV; h += blockDim.x) {
+      const int hx = h % HX, t = h / HX, hy = t % HY, hz = t / HY;
+      const int gz = z0 - 1 + hz, gy = y0 - 1 + hy, gx = x0 - 1 + hx;
+      s_h[t * HXP + hx] = inside(d, gz, gy, gx) ? __bfloat162float(a0[vox(d, gz, gy, gx)]) : 0.f;
+    }
     for (int i = threadIdx.x; i < TV * 4; i += blockDim.x) {
       const int c = i & 3, r = i >> 2;
       const int gz = z0 + (r >> 7), gy = y0 + ((r >> 4) & 7), gx = x0 + (r & 15);
@@ -990,30 +1006,39 @@ k_wgrad_first(const bf16* __restrict__ a0, const bf16* __restrict__ g1, float* _
     }
     __syncthreads();
 #pragma unroll 1
-    for (int row = 0; row < TZ * TY; ++row) {
-      const int tz = row >> 3, ty = row & 7;
-      const float* hr = s_h + ((tz + kz) * HY + ty + ky) * HX;
-      const float* gr = s_g + row * TX * C + co;
-      float w0 = hr[0], w1 = hr[1];
-#pragma unroll 4
-      for (int tx = 0; tx < TX; ++tx) {
-        const float w2 = hr[tx + 2], g = gr[tx * C];
-        acc0 = fmaf(g, w0, acc0);
-        acc1 = fmaf(g, w1, acc1);
-        acc2 = fmaf(g, w2, acc2);
-        bacc += g;
-        w0 = w1;
-        w1 = w2;
+    for (int i = 0; i < 8; ++i) {                    // two rows of four chunks of four voxels
+      const int row = 2 * warp + (i >> 2), x = 4 * (i & 3), tz = row >> 3, ty = row & 7;
+      float g[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        g[e] = s_g[(row * TX + x + e) * C + co];
+        bacc += g[e];
+      }
+#pragma unroll
+      for (int r = 0; r < 9; ++r) {
+        const float* hr = s_h + ((tz + r / 3) * HY + ty + r % 3) * HXP + x;
+        const float4 p = *reinterpret_cast<const float4*>(hr), q = *reinterpret_cast<const float4*>(hr + 4);
+        const float v[6] = {p.x, p.y, p.z, p.w, q.x, q.y};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+          for (int kx = 0; kx < 3; ++kx) acc[3 * r + kx] = fmaf(g[e], v[e + kx], acc[3 * r + kx]);
       }
     }
   }
-  float* pp = part + (size_t)blockIdx.x * (NTAP * C) + (kz * 9 + ky * 3) * C + co;
-  pp[0] = acc0;
-  pp[C] = acc1;
-  pp[2 * C] = acc2;
-  if (kzy == 0) bpart[(size_t)blockIdx.x * C + co] = bacc;
+  // the eight warps' sums: [warp][28][32] in s_g, added in order
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < NTAP; ++t) s_g[(warp * (NTAP + 1) + t) * C + co] = acc[t];
+  s_g[(warp * (NTAP + 1) + NTAP) * C + co] = bacc;
+  __syncthreads();
+  for (int i = threadIdx.x; i < (NTAP + 1) * C; i += blockDim.x) {
+    float t = 0.f;
+    for (int v = 0; v < 8; ++v) t += s_g[v * (NTAP + 1) * C + i];
+    if (i < NTAP * C) part[(size_t)blockIdx.x * (NTAP * C) + i] = t;
+    else bpart[(size_t)blockIdx.x * C + i - NTAP * C] = t;
+  }
 }
-
 
 // ------------------------------------------------------------------ reductions, input, parameters
 
@@ -1406,9 +1431,9 @@ void forward_to_a5(muffin_net* n, const float* y) {
   k_scale_final<<<1, 32, 0, n->st>>>(n->mpart, grid_s, n->s);
   const int grid_p = (int)((d.nvox + 255) / 256 < 4 * n->sms ? (d.nvox + 255) / 256 : 4 * n->sms);
   k_prep_input<<<grid_p, 256, 0, n->st>>>(y, n->s, n->a0, d.nvox);
-  const int gsimt = d.ntiles < 4 * n->sms ? d.ntiles : 4 * n->sms;
+  const int gsimt = d.ntiles < 5 * n->sms ? d.ntiles : 5 * n->sms;   // five blocks an SM
   bf16* out = n->map(0);
-  k_first_fwd<<<gsimt, 256, 0, n->st>>>(n->a0, n->kw.w1, n->kw.b1, out, d);
+  k_first_fwd<<<gsimt, kFirstThreads, 0, n->st>>>(n->a0, n->kw.w1, n->kw.b1, out, d);
   for (int l = 0; l < 4; ++l) {
     bf16* in = out;
     out = n->training ? n->map(l + 1) : n->map((l + 1) & 1);
@@ -1467,8 +1492,8 @@ void loss_and_grad(muffin_net* n, const float* y, const float* tx, const bf16* t
     bf16* tmp = g; g = other; other = tmp;
   }
   int P = part_slots(d);
-  if (P > 2 * n->sms) P = 2 * n->sms;
-  k_wgrad_first<<<P, 288, 0, n->st>>>(n->a0, g, n->part, n->bpart, d);
+  if (P > 3 * n->sms) P = 3 * n->sms;      // three blocks an SM
+  k_wgrad_first<<<P, 256, 0, n->st>>>(n->a0, g, n->part, n->bpart, d);
   launch_reduce(n->part, P, NTAP * C, n->grad + w_offset(0), MAP_FIRST, 1, n->bpart, n->grad + b_offset(0, n->K), n->st);
 }
 
