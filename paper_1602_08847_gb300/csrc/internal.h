@@ -99,6 +99,10 @@ bool iuwt_march_adjoint(const Geom& g);
 cudaError_t launch_fine_analysis_march(const Geom& g, const IuwtArgs& a, cudaStream_t s);
 cudaError_t launch_fine_adjoint_march(const Geom& g, const IuwtArgs& a, cudaStream_t s);
 cudaError_t iuwt_march_configure(const Geom& g);
+// The coarse levels as a march of single warps (k_coarse_march.cu).
+bool coarse_march_ok(const Geom& g);
+cudaError_t launch_coarse_march(const Geom& g, const float* c_in, float* r_out, float* U, float k, float rho,
+                                cudaStream_t s);
 cudaError_t fft_configure(int n);
 
 // ---- W_s as a union of eight orthonormal Daubechies bases (k_dwt.cu) ----

@@ -973,6 +973,10 @@ static cudaError_t coarse_n(const Geom& g, const float* c_in, float* r_out, floa
 
 cudaError_t launch_coarse(const Geom& g, const float* c_in, float* r_out, float* U, float k, float rho, int mode,
                           double* partials, cudaStream_t s, int* nblocks) {
+  if (mode == MODE_UPDATE && coarse_march_ok(g)) {
+    if (nblocks) *nblocks = (1 << (2 * g.j1)) * g.L;
+    return launch_coarse_march(g, c_in, r_out, U, k, rho, s);
+  }
   if (g.vec && mode == MODE_UPDATE && iuwt_vec_coarse_ok(g)) {
     if (nblocks) *nblocks = (1 << (2 * g.j1)) * g.L;
     return launch_coarse_vec(g, c_in, r_out, U, k, rho, s);

@@ -1,4 +1,5 @@
-"""The row march of the fine wavelet levels (large cubes) against the general
+"""The row march of the fine wavelet levels (large cubes) and of the coarse
+levels on 128 x 128 sub-images (512 of them at least) against the general
 kernels, which the same cube runs on when MUFFIN_IUWT_GENERAL is set: every
 width, split and level count the march takes, the coarse plane's dual in its
 epilogue (J = j1), relaxation, strips that end inside a channel, and channel
@@ -11,6 +12,9 @@ pytestmark = pytest.mark.gpu
 # (n, L, J, j1): at least 2^22 pixels unless noted
 CASES = [(128, 257, 3, 1), (128, 256, 3, 2), (128, 259, 3, 3), (128, 258, 4, 3), (256, 67, 1, 1), (256, 65, 4, 2),
          (256, 64, 3, 3), (512, 17, 2, 2), (512, 33, 5, 3), (1024, 4, 3, 3), (1024, 5, 4, 3),
+         (1024, 8, 4, 3), (1024, 9, 5, 3),       # coarse march too
+         (1024, 7, 5, 3),                       # too few sub-images for it
+         (64, 9, 3, 0), (32, 5, 2, 0), (64, 64, 1, 0),      # the whole image as one resident sub-image
          (256, 33, 4, 2),                       # march adjoint, tile analysis
          (256, 31, 4, 2), (512, 7, 4, 3)]       # below both thresholds
 
