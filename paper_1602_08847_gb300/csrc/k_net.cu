@@ -1363,6 +1363,7 @@ struct muffin_net {
   bf16* act = nullptr;   // training: a1..a5; inference: two ping-pong maps
   bf16* gA = nullptr;
   bf16* gB = nullptr;
+  bf16* d6 = nullptr;    // loss gradient, split (split3)
 
   bf16* map(int i) const { return act + (size_t)i * d.nvox * C; }
 };
@@ -1403,10 +1404,11 @@ size_t net_layout(muffin_net* n, const Dims& d, int K, int training, char* base)
   bf16* act = (bf16*)take((training ? 5 : 2) * V * C * 2);
   bf16* gA = (bf16*)take(training ? V * C * 2 : 0);
   bf16* gB = (bf16*)take(training ? V * C * 2 : 0);
+  bf16* d6 = (bf16*)take(training ? V * C * 2 : 0);
   if (n) {
     n->theta = theta; n->mom1 = m1; n->mom2 = m2; n->grad = grad; n->kw = kw;
     n->s = s; n->mpart = mpart; n->lpart = lpart; n->loss = loss; n->part = part; n->bpart = bpart;
-    n->a0 = a0; n->act = act; n->gA = gA; n->gB = gB;
+    n->a0 = a0; n->act = act; n->gA = gA; n->gB = gB; n->d6 = d6;
   }
   return off;
 }
@@ -1458,11 +1460,12 @@ void last_predict(muffin_net* n, float* x, float* aux) {
   launch_tc05<EPI_PRED>(a5_of(n), n->kw.w6t, n->kw.b6, nullptr, nullptr, n->d, n->sms, n->st, la);
 }
 
-// Last layer of the training pass: loss, its gradient d6 (into a map, split),
+// Last layer of the training pass: loss, its gradient d6 (split),
 // the layer's weight and bias gradients, and the gradient of a5's
 // pre-activation into g5.
-void last_train(muffin_net* n, const float* tx, const bf16* taux, bf16* d6, bf16* g5) {
+void last_train(muffin_net* n, const float* tx, const bf16* taux, bf16* g5) {
   const Dims& d = n->d;
+  bf16* d6 = n->d6;
   bf16* a5 = a5_of(n);
   LastArgs la = last_args(n);
   la.tx = tx;
@@ -1483,7 +1486,7 @@ void loss_and_grad(muffin_net* n, const float* y, const float* tx, const bf16* t
   forward_to_a5(n, y);
   bf16* g = n->gA;
   bf16* other = n->gB;
-  last_train(n, tx, taux, other, g);      // `other` holds d6 until the first layer gradient overwrites it
+  last_train(n, tx, taux, g);
   for (int k = 4; k >= 1; --k) {          // layers 5..2 (index k), input map a_k = map(k - 1)
     const bf16* a_in = n->map(k - 1);
     launch_wgrad_mid(a_in, g, n->part, n->bpart, n->grad + w_offset(k), n->grad + b_offset(k, n->K), d, n->sms,
