@@ -24,7 +24,6 @@
 // bound), adjoint 670 -> 286 (1.34 GB: 4.7 TB/s; 12 warps per SM, bound by the
 // latency and the issue slots of a step).  256 x 256 x 64, two levels: 28.7 ->
 // 22.8 and 40.9 -> 21.0.
-#include <cstdlib>
 
 #include "internal.h"
 #include "iuwt_vec.cuh"

