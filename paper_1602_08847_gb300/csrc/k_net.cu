@@ -1044,10 +1044,11 @@ k_wgrad_first(const bf16* __restrict__ a0, const bf16* __restrict__ g1, float* _
 
 enum { MAP_MID = 1, MAP_FIRST = 2, MAP_LAST = 3 };
 
-// sum_b p[b * n], b = 0 .. P-1, in that order, eight loads in flight: the loop
-// is one load latency per trip (a 31x120x100 layer's weight gradient took 99.7
-// us with four loads a trip and blocks of 256, 79.5 so, in blocks of 64 and
-// with the biases in the same launch).
+// sum_b p[b * n], b = 0 .. P-1, eight at a time in flight: the loop is one load
+// latency per trip (a 31x120x100 layer's weight gradient took 99.7 us with four
+// loads a trip and blocks of 256, 79.5 so, in blocks of 64 and with the biases
+// in the same launch).  The eight are added as a float pair, then to the double
+// (with a conversion and an addition in FP64 for each the call takes 79.5 us, so 72.1).
 __device__ __forceinline__ double sum_parts(const float* __restrict__ p, int P, size_t n) {
   double s = 0.0;
   int b = 0;
@@ -1055,8 +1056,15 @@ __device__ __forceinline__ double sum_parts(const float* __restrict__ p, int P, 
     float v[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[e] = p[(size_t)(b + e) * n];
+    Pair t{0.f, 0.f};
 #pragma unroll
-    for (int e = 0; e < 8; ++e) s += v[e];
+    for (int e = 0; e < 8; ++e) t.add(v[e], 0.f);
+    if (fabsf(t.hi) <= 1e37f && fabsf(t.lo) <= 1e37f) {
+      s += (double)t.hi + (double)t.lo;
+    } else {                         // infinities, NaN, or sums near the end of the range
+#pragma unroll 1
+      for (int e = 0; e < 8; ++e) s += p[(size_t)(b + e) * n];
+    }
   }
   for (; b < P; ++b) s += p[(size_t)b * n];
   return s;
