@@ -218,10 +218,10 @@ struct Pair {
 // Weights are [shift][chunk][2 - kz][co][16 B] (next 8 outputs 128 B, next 8
 // inputs 1536 B), loaded once per CTA.
 //
-// Every wait is bounded: a role that gives up records it in g_tc_timeouts and
-// leaves, the others run into their own bounds, and the CTA waits for its
-// copies and MMAs in flight (at the full bound) before it frees its tensor
-// memory.
+// Every wait is bounded: a warp that gives up (all of its lanes together:
+// warp_wait) records it in g_tc_timeouts and leaves, the others run into their
+// own bounds, and the CTA waits for its copies and MMAs in flight (at the full
+// bound) before it frees its tensor memory.
 constexpr int U_TY = 16, U_TX = 8;                          // output tile: 16 rows x 8 columns, one channel
 constexpr int U_HY = U_TY + 2, U_HX = U_TX + 2;             // 18 x 10 halo of a plane
 constexpr int Z_CH = 2976;                                  // chunk pitch of a plane slot (180 voxels x 16 B, padded)
@@ -274,6 +274,13 @@ __device__ __forceinline__ bool mbar_wait_n(uint32_t bar, uint32_t parity, long 
 // stood in front of every poll).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long long polls) {
   return mbar_wait_n(bar, parity, polls);
+}
+// The same for a whole warp, as one decision: its lanes poll on their own and
+// may see the bound run out differently, and a lane that left alone would let
+// the others run the warp's aligned tcgen05 loads, or wait in a full-mask vote,
+// without it.  The vote also brings the lanes together again.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, long long polls) {
+  return __all_sync(0xffffffffu, mbar_wait_n(bar, parity, polls));
 }
 // drain wait after a give-up: the full bound
 __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity) { return mbar_wait_n(bar, parity, kWaitLimit); }
@@ -343,6 +350,7 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
     muffin::mbar_init(s_fin, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  __syncwarp();
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(s_tm) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -395,7 +403,7 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
       }
       for (int z = za - 1; z <= zb; ++z) {
         const int slot = np % Z_NS;
-        if (!mbar_wait(s_free + 8 * slot, (uint32_t)(np / Z_NS & 1) ^ 1u, polls)) { ok = false; break; }
+        if (!warp_wait(s_free + 8 * slot, (uint32_t)(np / Z_NS & 1) ^ 1u, polls)) { ok = false; break; }
         const bool in_z = (unsigned)z < (unsigned)d.nz;
         const unsigned char* pl = base + (in_z ? (size_t)z * pitch : 0);
         const uint32_t sp = s0 + slot * Z_PLANE;
@@ -507,7 +515,7 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
               if (k < la.K) tk[k] = __bfloat162float(ta[(size_t)(k - 1) * plane]);
           }
         }
-        if (!mbar_wait(s_done + 8 * acc, (uint32_t)(no / Z_RING & 1), polls)) { ok = false; break; }
+        if (!warp_wait(s_done + 8 * acc, (uint32_t)(no / Z_RING & 1), polls)) { ok = false; break; }
         tc_fence_after();
         const uint32_t taddr = tmem + (uint32_t)(acc * NO) + ((uint32_t)(warp * 32) << 16);
         if constexpr (!kLast) {
@@ -603,6 +611,7 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
   tc_fence_before();
   if (__syncthreads_or(!ok || !fin) && threadIdx.x == 0) atomicAdd(&g_tc_timeouts, 1);
   tc_fence_after();
+  __syncwarp();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
   if constexpr (EPI == EPI_LOSS) {
     // lpart[block] = (sum_k lam_k sum_p r_k^2, sum_p r_0, ..., sum_p r_{K-1}), fixed order
@@ -691,6 +700,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
     muffin::mbar_init(s_go, 96);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  __syncwarp();
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(s_tm) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -702,6 +712,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(s_tm) : "memory");
   auto clear = [&] {                            // warps 0-3: this warp's lanes of the accumulators
     const uint32_t ta = tmem + ((uint32_t)(warp * 32) << 16);
+    __syncwarp();
     for (int c = 0; c < 3 * WG_N; c += 8)
       asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(ta + (uint32_t)c),
                    "r"(0u)
@@ -716,6 +727,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
     for (int q = 0; q < 18; ++q) {            // (kx, 2 - kz) = q / 2, columns (co) 16 (q % 2) .. + 15
       const int acc = q >> 1, co0 = (q & 1) * 16, kx = acc / 3, kz = 2 - acc % 3;
       uint32_t r[16];
+      __syncwarp();
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
           : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
@@ -782,7 +794,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
       }
       for (int i = 0; i < n + 2; ++i) {
         const int slot = np % WG_NS, z = za - 1 + i;
-        if (!mbar_wait(s_free + 8 * slot, (uint32_t)(np / WG_NS & 1) ^ 1u, polls)) { ok = false; break; }
+        if (!warp_wait(s_free + 8 * slot, (uint32_t)(np / WG_NS & 1) ^ 1u, polls)) { ok = false; break; }
         const bool in_z = (unsigned)z < (unsigned)d.nz;
         const unsigned char* pl = pa + (in_z ? (size_t)z * pitch : 0);
         const uint32_t sp = s0 + slot * WG_A;
@@ -860,7 +872,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
       const int n = zb - za;
       for (int i = 0; i < n + 2; ++i) {
         const int slot = np % WG_NS;
-        if (!mbar_wait(s_full + 8 * slot, (uint32_t)(np / WG_NS & 1), polls)) { ok = false; break; }
+        if (!warp_wait(s_full + 8 * slot, (uint32_t)(np / WG_NS & 1), polls)) { ok = false; break; }
         if (i < n) {
           const unsigned char* t = base + ((no + i) % WG_R) * (4 * U_TX * 16) + c * U_TX * 16;
 #pragma unroll
@@ -875,8 +887,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
         mbar_arrive(s_free + 8 * slot);
         ++np;
         if (flush > 0 && np % flush == 0 && warp < 3) {
-          const bool stopped = mbar_wait(s_stop, (uint32_t)(np / flush - 1) & 1u, polls);
-          if (!__all_sync(0xffffffffu, stopped)) { ok = false; break; }
+          if (!warp_wait(s_stop, (uint32_t)(np / flush - 1) & 1u, polls)) { ok = false; break; }
           tc_fence_after();
           store(flushed, false);
           flushed = true;
@@ -906,6 +917,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  __syncwarp();
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
