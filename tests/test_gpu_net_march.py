@@ -1,5 +1,7 @@
 """The marching tensor-core kernels of the network (k_net.cu): waits that run
-out part of the way, at poll bounds between none and enough."""
+out part of the way, at poll bounds between none and enough; and the kernels'
+steady state (many tiles a block: full rings, every barrier phase, runs that
+cross columns) on integers, where every result is exact."""
 import pytest
 import torch
 
@@ -54,3 +56,122 @@ def test_waits_that_run_out_midway(netmod, polls):
         assert all(torch.equal(p, q) for p, q in zip(f(), ref))
         assert netmod.wait_timeouts() == 0
     n.close()
+
+
+# ---------------------------------------------------------------- exact references
+#
+# Small integers throughout: every product and every sum of the kernels is an
+# integer (times a power of two) below 2^24, exact in float32 whatever the order
+# and the rounding of the additions, so results are compared for equality.  The
+# one rounding left, of a map to bfloat16, is to nearest even on both sides.
+
+SHAPES = [(40, 20, 20),        # few tall columns: one tile a block
+          (31, 120, 100),      # 3224 tiles of the layers: eleven a block (21 in the weight gradient), ragged edges
+          (64, 200, 136),      # 14144: runs of 46 (93), whole columns and parts of two
+          (3, 264, 520)]       # 3315, columns shorter than the rings
+
+
+def ints(shape, seed, lo, hi, keep=1.0):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    v = torch.randint(lo, hi + 1, shape, device="cuda", generator=g).double()
+    return v if keep == 1.0 else v * (torch.rand(shape, device="cuda", generator=g) < keep)
+
+
+def windows(a):
+    """The 27 zero-padded shifts of a [z][y][x][f] map, each as a matrix."""
+    z, y, x, f = a.shape
+    ap = torch.nn.functional.pad(a, (0, 0, 1, 1, 1, 1, 1, 1))
+    for t in range(27):
+        kz, ky, kx = t // 9, t // 3 % 3, t % 3
+        yield t, ap[kz:kz + z, ky:ky + y, kx:kx + x].reshape(-1, f)
+
+
+def conv(a, w, b=None):
+    w = w.reshape(*w.shape[:2], 27)
+    out = torch.zeros(a[..., 0].numel(), w.shape[0], dtype=torch.float64, device="cuda")
+    for t, m in windows(a):
+        out.addmm_(m, w[:, :, t].T)
+    out = out.reshape(*a.shape[:3], -1)
+    return out if b is None else out + b
+
+
+def conv_back(dz, w):
+    return conv(dz, w.transpose(0, 1).flip(2, 3, 4))
+
+
+def conv_weights(a, dz):
+    d = dz.reshape(-1, dz.shape[-1])
+    dw = torch.stack([d.T @ m for _, m in windows(a)], dim=2)
+    return dw.reshape(*dw.shape[:2], 3, 3, 3), d.sum(0)
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_layers_exact(netmod, shape):
+    a, dz = ints(shape + (32,), 1, 0, 2), ints(shape + (32,), 2, -2, 2)
+    w, b = ints((32, 32, 3, 3, 3), 3, -3, 3), ints((32,), 4, -9, 9)
+    assert 2 * 2 * a[..., 0].numel() < 2 ** 24
+    A, D, W, B = a.bfloat16(), dz.bfloat16(), w.float(), b.float()
+    z = conv(a, w, b)
+    assert torch.equal(netmod.conv3d_forward(A, W, B, True), z.clamp(min=0).bfloat16())
+    assert torch.equal(netmod.conv3d_forward(A, W, None, False), (z - b).bfloat16())
+    da = conv_back(dz, w)
+    assert torch.equal(netmod.conv3d_backward_data(D, W, None), da.bfloat16())
+    assert torch.equal(netmod.conv3d_backward_data(D, W, A), (da * (a > 0)).bfloat16())
+    dw, db = conv_weights(a, dz)
+    got_w, got_b = netmod.conv3d_backward_weights(A, D)
+    assert torch.equal(got_w, dw.float()) and torch.equal(got_b, db.float())
+    assert netmod.wait_timeouts() == 0
+
+
+def sparse_weights(co, ci, seed, per_row=3):
+    """+-1 at per_row places of each output's 27 ci weights."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    w = torch.zeros(co, ci * 27, dtype=torch.float64, device="cuda")
+    at = torch.rand(co, ci * 27, device="cuda", generator=g).argsort(dim=1)[:, :per_row]
+    sign = 2.0 * torch.randint(0, 2, at.shape, device="cuda", generator=g).double() - 1.0
+    return w.scatter_(1, at, sign).reshape(co, ci, 3, 3, 3)
+
+
+@pytest.mark.parametrize("shape,K", [((64, 100, 64), 1), ((64, 100, 64), 6), ((31, 120, 100), 8), ((7, 264, 264), 3)])
+def test_network_exact(netmod, shape, K):
+    """Prediction, loss and gradient: maps of integers of at most 3^5, from a sparse cube of zeros and ones and three
+    weights of +-1 an output; loss weights that make the factor of the loss gradient a power of two."""
+    V = shape[0] * shape[1] * shape[2]
+    layers = [(sparse_weights(co, ci, 50 + i), torch.zeros(co, dtype=torch.float64, device="cuda"))
+              for i, (ci, co) in enumerate([(1, 32)] + [(32, 32)] * 4 + [(32, K)])]
+    theta = torch.cat([t.reshape(-1) for wb in layers for t in wb]).float()
+    lam = [V / 2.0 ** (2 + k % 3) for k in range(K)]       # 2 / V lam = 2^-1, 2^-2, 2^-3
+    y = ints(shape, 60, 1, 1, keep=0.03)
+    tx = ints(shape, 61, 0, 3, keep=0.03)
+    ta = ints((shape[0], K - 1) + shape[1:], 62, -1, 1, keep=0.03) if K > 1 else None
+    assert float(y.max()) == 1.0
+    acts = [y[..., None]]
+    for i, (w, b) in enumerate(layers):
+        z = conv(acts[-1], w, b)
+        acts.append(z.clamp(min=0).bfloat16().double() if i < 5 else z)
+    net = netmod.WarmStartNet(shape, theta=theta, n_out=K, out_weight=lam)
+    x, aux = net.predict(y.float())
+    assert torch.equal(x, acts[-1][..., 0].clamp(min=0).float())
+    if K > 1:
+        assert torch.equal(aux, acts[-1][..., 1:].clamp(-1, 1).permute(0, 3, 1, 2).float())
+    net.close()
+    target = tx[..., None] if ta is None else torch.cat([tx[..., None], ta.permute(0, 2, 3, 1)], dim=-1)
+    r = acts[-1] - target
+    L = torch.tensor(lam, dtype=torch.float64, device="cuda")
+    loss = float((L * r * r).sum()) / V
+    dz, grads = torch.tensor([2.0 * v / V for v in lam], dtype=torch.float64, device="cuda") * r, []   # powers of two
+    for i in range(5, -1, -1):
+        dw, db = conv_weights(acts[i], dz)
+        # the premise: every sum of magnitudes stays below 2^24 units of 2^-3 (one unit of the loss gradient)
+        mw, mb = conv_weights(acts[i].abs(), dz.abs())
+        assert max(float(mw.max()), float(mb.max())) * 8 < 2 ** 24
+        grads = [dw.reshape(-1), db] + grads
+        if i:
+            dz = (conv_back(dz, layers[i][0]) * (acts[i] > 0)).bfloat16().double()
+    net = netmod.WarmStartNet(shape, training=True, theta=theta, n_out=K, out_weight=lam)
+    got, g = net.loss_grad(y.float(), tx.float(), None if ta is None else ta.bfloat16().contiguous())
+    assert got == loss
+    want = torch.cat(grads).float()
+    assert float(want.abs().max()) > 0 and torch.equal(g, want)
+    net.close()
+    assert netmod.wait_timeouts() == 0
