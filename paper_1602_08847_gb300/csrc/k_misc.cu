@@ -2,6 +2,7 @@
 // a counter-based start vector, and the plane permutation between the natural
 // and the class-permuted layouts of U.
 #include "device.cuh"
+#include "exact_sum.cuh"
 #include "internal.h"
 
 namespace muffin {
@@ -30,10 +31,11 @@ __global__ void __launch_bounds__(1024) k_reduce_partials(const double* __restri
 // FP64 runs at 1/64 of the FP32 rate here: the conversions and the double
 // multiply-add of every value, and a square root and division in every thread
 // of the scaling, bound these two kernels of the power method at 410 and 400 us
-// for 67 M values; 60 and 80 us so.  Products are split exactly into
-// two floats and summed in float pairs (Knuth's two-sum) over 16 values, then
-// added to the double; a group with a product outside the range in which that
-// is exact is summed in double.
+// for 67 M values; 95 and 80 us so.  Products are split exactly into
+// two floats and summed in three floats (Sum3) over 16 values, then added to the
+// double: three roundings to double where every value had one (float pairs, 60 us,
+// lost the bits past 48).  A group with a
+// product outside the range in which that is exact is summed in double.
 __global__ void __launch_bounds__(256) k_dot(const float* __restrict__ a, const float* __restrict__ b, size_t n,
                                             double* partials) {
   __shared__ double red[32];
@@ -53,18 +55,16 @@ __global__ void __launch_bounds__(256) k_dot(const float* __restrict__ a, const 
       x[4 * e] = u.x; x[4 * e + 1] = u.y; x[4 * e + 2] = u.z; x[4 * e + 3] = u.w;
       y[4 * e] = v.x; y[4 * e + 1] = v.y; y[4 * e + 2] = v.z; y[4 * e + 3] = v.w;
     }
-    float hi = 0.f, lo = 0.f;
+    Sum3 s;
     bool exact = true;
 #pragma unroll
     for (int e = 0; e < 16; ++e) {
-      const float p = x[e] * y[e], m = fabsf(p), t = hi + p, c = t - hi;
+      const float m = fabsf(__fmul_rn(x[e], y[e]));
       exact = exact && ((m >= 1e-28f && m <= 1e30f) || x[e] == 0.f || y[e] == 0.f);
-      lo += ((hi - (t - c)) + (p - c)) + fmaf(x[e], y[e], -p);
-      hi = t;
+      s.add_product(x[e], y[e]);
     }
     if (exact) {
-      acc += (double)hi;
-      acc += (double)lo;
+      s.into(acc);
     } else {
 #pragma unroll 1
       for (int e = 0; e < 4; ++e) {

@@ -1,0 +1,73 @@
+"""The long sums of the power method (k_misc.cu), called through the library's
+internal launchers: on integers a double holds every partial sum exactly, and
+so must the sums in floats between two additions to a double."""
+import ctypes
+import math
+
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+_P, _S = ctypes.c_void_p, ctypes.c_size_t
+
+
+def stream():
+    return torch.cuda.current_stream().cuda_stream
+
+
+def dot(lib, a, b):
+    """The partial sums of k_dot, added on the host (without rounding where they are finite)."""
+    f = lib.lib._ZN6muffin10launch_dotEPKfS1_mPdPiP11CUstream_st     # muffin::launch_dot
+    f.argtypes, f.restype = [_P, _P, _S, _P, ctypes.POINTER(ctypes.c_int), _P], ctypes.c_int
+    parts, np = torch.zeros(1024, dtype=torch.float64, device="cuda"), ctypes.c_int()
+    assert f(a.data_ptr(), b.data_ptr(), a.numel(), parts.data_ptr(), ctypes.byref(np), stream()) == 0
+    parts = parts[:np.value].tolist()
+    return math.fsum(parts) if all(map(math.isfinite, parts)) else sum(parts)
+
+
+def place(t, offset):
+    """t on the GPU, `offset` floats past a 16-byte boundary."""
+    buf = torch.zeros(t.numel() + 8, device="cuda")
+    out = buf[offset:offset + t.numel()]
+    out.copy_(t)
+    return out
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 16, 17, 115, 1027, 4096, 4099])
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("lo", [-1, 0])          # both signs, and one
+def test_dot_is_exact_where_doubles_are(lib, n, offset, lo):
+    g = torch.Generator().manual_seed(100 * n + offset)
+    # at most 115 products that are not zero, so every partial sum is below 115 * 2^46 < 2^53; in the long ones they
+    # are the 16 products of each of the first threads: float4 t + 256 e of a block of 256 threads
+    keep = torch.arange(n) if n <= 115 else torch.tensor([4 * (t + 256 * e) + c for t in range(7) for e in range(4)
+                                                          for c in range(4) if 4 * (t + 256 * e) + c < n])
+    for _ in range(20):
+        a, b = torch.zeros(n, dtype=torch.int64), torch.zeros(n, dtype=torch.int64)
+        a[keep] = torch.randint(lo * 2 ** 23 + 1, 2 ** 23, (len(keep),), generator=g)
+        b[keep] = torch.randint(lo * 2 ** 23 + 1, 2 ** 23, (len(keep),), generator=g)
+        exact = sum(x * y for x, y in zip(a.tolist(), b.tolist()))
+        assert dot(lib, place(a.float(), offset), place(b.float(), offset)) == exact
+
+
+@pytest.mark.parametrize("offset", [0, 3])
+def test_dot_long_and_out_of_range(lib, offset):
+    g = torch.Generator().manual_seed(7)
+    n = (1 << 20) + 5
+    a, b = torch.randn(n, generator=g), torch.randn(n, generator=g)
+    scale = torch.ones(n)
+    scale[1000:3000] = 2.0 ** -80            # products below the range in which their errors are floats
+    scale[5000:5100] = 2.0 ** 50             # and sums near its end
+    a *= scale
+    b *= scale
+    terms = (a.double() * b.double()).tolist()
+    exact = math.fsum(terms)
+    got = dot(lib, place(a, offset), place(b, offset))
+    # at most ceil(n / 2^18) = 5 values or groups a thread (one a group in the unaligned case), three additions a group,
+    # five levels of a warp and five of a block, each rounding to 2^-53 of a sum of at most the magnitudes
+    assert abs(got - exact) <= 32 * 2.0 ** -53 * math.fsum(abs(t) for t in terms)
+    for bad, check in ((float("inf"), math.isinf), (float("nan"), math.isnan)):
+        a[777] = bad
+        b[777] = 1.0
+        assert check(dot(lib, place(a, offset), place(b, offset)))
