@@ -1,6 +1,7 @@
-// Sums of floats between two additions to a double.  Double arithmetic runs at
-// 1/64 of the float rate here, so long sums add a few terms in floats first; by
-// error-free steps, so that no bit is lost that a double would have held.
+// Double results by float arithmetic.  Double arithmetic runs at 1/64 of the
+// float rate here, so long sums add a few terms in floats between two additions
+// to a double, by error-free steps, so that no bit is lost that a double would
+// have held; and a product that is rounded to float in the end is formed in two.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -40,5 +41,21 @@ struct Sum3 {
     acc += (double)lo;
   }
 };
+
+// (float)((double)x * f) without double arithmetic, for f = hi + lo to 2^-48 of
+// itself and 1e-30 <= hi <= 1e30: x f is formed in two floats, p + t, with an
+// error below 2^-24 |t| + 2^-47 |p|; where p + (t - w) and p + (t + w) round to
+// the same float for twice that as w, so does x f, and so does x f rounded to
+// double first.  False where they differ (7 values in 10^7) or a term leaves the
+// range of floats.
+__device__ __forceinline__ bool scale_float(float x, float hi, float lo, float* out) {
+  const float p = __fmul_rn(x, hi), m = fabsf(p);
+  const float t = __fmaf_rn(x, lo, __fmaf_rn(x, hi, -p));
+  const float w = __fmaf_rn(m, 0x1p-46f, fabsf(t) * 0x1p-22f);
+  const float a = __fadd_rn(p, __fsub_rn(t, w)), b = __fadd_rn(p, __fadd_rn(t, w));
+  *out = a;
+  if (x == 0.f) *out = x;
+  return x == 0.f || (a == b && m >= 0x1p-90f && m <= 0x1p120f);
+}
 
 }  // namespace muffin

@@ -30,12 +30,12 @@ __global__ void __launch_bounds__(1024) k_reduce_partials(const double* __restri
 
 // FP64 runs at 1/64 of the FP32 rate here: the conversions and the double
 // multiply-add of every value, and a square root and division in every thread
-// of the scaling, bound these two kernels of the power method at 410 and 400 us
-// for 67 M values; 95 and 80 us so.  Products are split exactly into
-// two floats and summed in three floats (Sum3) over 16 values, then added to the
-// double: three roundings to double where every value had one (float pairs, 60 us,
-// lost the bits past 48).  A group with a
-// product outside the range in which that is exact is summed in double.
+// of the scaling, bound these two kernels of the power method at 404 and 406 us
+// for 67 M values; 95 and 90 us so.  Products are split exactly into two floats
+// and summed in three (Sum3) over 16 values, then added to the double: three
+// roundings to double where every value had one (float pairs, 60 us, lost the
+// bits past 48).  A group with a product outside the range in which that is
+// exact is summed in double.
 __global__ void __launch_bounds__(256) k_dot(const float* __restrict__ a, const float* __restrict__ b, size_t n,
                                             double* partials) {
   __shared__ double red[32];
@@ -79,8 +79,13 @@ __global__ void __launch_bounds__(256) k_dot(const float* __restrict__ a, const 
   if (threadIdx.x == 0) partials[blockIdx.x] = acc;
 }
 
-// x <- x * num / sqrt(den)   (num == nullptr: factor 1); the factor, formed
-// once a block, as two floats where it has them
+__device__ __noinline__ float4 scale4_double(float4 v, double f) {   // a call: seldom taken
+  return make_float4((float)(v.x * f), (float)(v.y * f), (float)(v.z * f), (float)(v.w * f));
+}
+
+// x <- (float)(x * num / sqrt(den))   (num == nullptr: factor 1); the factor is
+// formed once a block, and where it is two floats the values are rounded through
+// them (scale_float), the few it cannot tell in double.  67 M values: 90 us
 __global__ void k_scale(float* x, size_t n, const double* num, const double* den) {
   __shared__ double s_f;
   __shared__ float s_hi, s_lo;
@@ -98,9 +103,13 @@ __global__ void k_scale(float* x, size_t n, const double* num, const double* den
 #pragma unroll 2
     for (size_t i = first; i < n4; i += step) {
       const float4 v = x4[i];
-      x4[i] = make_float4(fmaf(v.x, hi, v.x * lo), fmaf(v.y, hi, v.y * lo), fmaf(v.z, hi, v.z * lo), fmaf(v.w, hi, v.w * lo));
+      float4 r;
+      const bool a = scale_float(v.x, hi, lo, &r.x), b = scale_float(v.y, hi, lo, &r.y);
+      const bool c = scale_float(v.z, hi, lo, &r.z), d = scale_float(v.w, hi, lo, &r.w);
+      if (!(a && b && c && d)) r = scale4_double(v, s_f);
+      x4[i] = r;
     }
-    for (size_t i = 4 * n4 + first; i < n; i += step) x[i] = fmaf(x[i], hi, x[i] * lo);
+    for (size_t i = 4 * n4 + first; i < n; i += step) x[i] = (float)(x[i] * s_f);
   } else {
     for (size_t i = first; i < n; i += step) x[i] = (float)(x[i] * s_f);
   }

@@ -1,4 +1,4 @@
-"""The long sums of the power method (k_misc.cu), called through the library's
+"""The long sums and the scaling of the power method (k_misc.cu), called through the library's
 internal launchers: on integers a double holds every partial sum exactly, and
 so must the sums in floats between two additions to a double."""
 import ctypes
@@ -71,3 +71,25 @@ def test_dot_long_and_out_of_range(lib, offset):
         a[777] = bad
         b[777] = 1.0
         assert check(dot(lib, place(a, offset), place(b, offset)))
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+def test_scale_rounds_the_double_product(lib, offset):
+    """x <- (float)((double)x * f) to the bit, for every significand and both paths of the kernel."""
+    fn = lib.lib._ZN6muffin12launch_scaleEPfmPKdS2_P11CUstream_st    # muffin::launch_scale
+    fn.argtypes, fn.restype = [_P, _S, _P, _P, _P], ctypes.c_int
+    one = torch.ones(1, dtype=torch.float64, device="cuda")
+    ordinary = (torch.arange(2 ** 23, dtype=torch.int32, device="cuda") + 0x3F800000).view(torch.float32)   # [1, 2)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    wild = torch.randint(-2 ** 31, 2 ** 31, (2 ** 20 + 3,), device="cuda", generator=g).int().view(torch.float32)
+    wild[:4] = torch.tensor([0.0, -0.0, float("inf"), float("-inf")])    # any bits: every exponent, NaNs among them
+    factors = [(0.5 + k / 23.0) ** 0.5 for k in range(12)] + [1.0, 0.25, 3.1e-5, 7.7e8]
+    factors += [1e-31, 3e-38, 1e-44, 1e31, 1e300, 0.0, float("inf"), float("nan")]   # factors without two floats
+    for x in (ordinary, wild):
+        for f in factors if x is wild else factors[:16]:
+            num = torch.tensor([f], dtype=torch.float64, device="cuda")
+            got = place(x, offset)
+            assert fn(got.data_ptr(), got.numel(), num.data_ptr(), one.data_ptr(), stream()) == 0
+            want = (x.double() * f).float()
+            same = (got.view(torch.int32) == want.view(torch.int32)) | (got.isnan() & want.isnan())
+            assert bool(same.all()), (f, x[~same][:3], got[~same][:3], want[~same][:3])
