@@ -301,6 +301,10 @@ struct Runs {
     at = total * blockIdx.x / gridDim.x;
     end = total * (blockIdx.x + 1) / gridDim.x;
   }
+  // input planes of the whole run: each stretch reads one before and one after its tiles
+  __device__ __forceinline__ int planes(int nz) const {
+    return at < end ? (int)(end - at + 2 * ((end - 1) / nz - at / nz + 1)) : 0;
+  }
   // next stretch za .. zb-1 of one column; false at the end
   __device__ __forceinline__ bool next(int nz, int& col, int& za, int& zb) {
     if (at >= end) return false;
@@ -631,13 +635,11 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
 // dz planes zi - 1, zi, zi + 1 at once (kz = 2, 1, 0), so one accumulator of
 // 128 x 96 per kx holds the nine row and channel offsets of its taps (rows
 // 96..127, "ky = 3", are computed and dropped).  The three accumulators (288
-// columns) stay in tensor memory for the CTA's whole run over its tiles; the
-// sums leave TMEM once, at the end, or every `flush` planes: the tensor core
-// adds with truncation, which over a run of 1700 additions of one sign costs
-// 1e-4 of the sum.  The 32 -> 32 layers' bfloat16 gradients carry that anyway;
-// the last layer's, whose operand is exact (split3), is flushed every 4 planes
-// (32 additions) onto float32 sums in shared memory, rounded to nearest.  24 MMAs of N = 96 per
-// tile replace 72 of N = 32; an MMA takes as long either way (the read of its A
+// columns) stay in tensor memory; every `flush` planes their sums are added to
+// float32 sums in shared memory, rounded to nearest, and they start over, since
+// the tensor core adds with truncation: a run of 1700 additions of one sign
+// loses 8e-5 of its sum (wgrad_flush has the rule).  24 MMAs of N = 96 per tile
+// replace 72 of N = 32; an MMA takes as long either way (the read of its A
 // operand).
 //
 // Both operands are MN-major (M or N contiguous: the 8 features of a chunk),
@@ -665,9 +667,9 @@ constexpr int WG_DROW = WG_R * 4 * U_TX * 16;          // row pitch of the ring 
 constexpr int WG_B = U_TY * WG_DROW;                   // 65536 B
 constexpr int WG_BAR = WG_NS * WG_A + WG_B;            // full, free, fin, TMEM slot
 constexpr int WG_SUM = 3 * 3 * C * 96 * 4;              // flushed sums, 110592 B
-// more than half an SM in any case: one CTA holds all of the tensor memory
-__host__ __device__ constexpr int wgrad05_smem(bool flush) { return flush ? WG_BAR + 256 + 128 + WG_SUM : 120 * 1024; }
-static_assert(WG_BAR + 256 + 128 <= wgrad05_smem(false) && wgrad05_smem(true) + 4096 <= muffin::kMaxDynSmem, "weight gradient shared memory");
+// more than half an SM: one CTA holds all of the tensor memory
+constexpr int wgrad05_smem = WG_BAR + 256 + 128 + WG_SUM;
+static_assert(wgrad05_smem + 4096 <= muffin::kMaxDynSmem, "weight gradient shared memory");
 constexpr int WG_N = 3 * C;
 constexpr int kLastFlush = 4;                          // planes between two flushes, last layer
 // D f32, A/B bf16, both MN-major, N = n, M = 128
@@ -719,7 +721,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
                    : "memory");
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
   };
-  // warps 0-2: the sums out of tensor memory, onto this CTA's flushed sums (s_sum, flush > 0), and at the end to part
+  // warps 0-2: the sums out of tensor memory, onto this CTA's flushed sums (s_sum), and at the end to part
   float* s_sum = reinterpret_cast<float*>(smem + (s0 - smem_u32(smem)) + WG_BAR + 256);
   auto store = [&](bool add, bool last) {
     // lane = ci, TMEM lanes 32 ky .. 32 ky + 31; columns kx * 96 + (2 - kz) * 32 + co
@@ -755,6 +757,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
 
   const long long polls = *(volatile long long*)&g_wait_polls;
   Runs runs(tiles_x * tiles_y, d.nz);
+  const int planes = runs.planes(d.nz);         // no flush after the last one: the sums leave then anyway
   int col, za, zb;
   bool ok = true;
   float bacc[8];
@@ -853,7 +856,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
         }
         tc_commit(s_free + 8 * slot);
         ++np;
-        if (flush > 0 && np % flush == 0) {
+        if (np % flush == 0 && np < planes) {
           tc_commit(s_stop);
           if (!mbar_wait(s_go, (uint32_t)(np / flush - 1) & 1u, polls)) { ok = false; break; }
           tc_fence_after();
@@ -886,7 +889,7 @@ k_wgrad_tc05(const bf16* __restrict__ a, const bf16* __restrict__ dz, float* __r
         }
         mbar_arrive(s_free + 8 * slot);
         ++np;
-        if (flush > 0 && np % flush == 0 && warp < 3) {
+        if (np % flush == 0 && np < planes && warp < 3) {
           if (!warp_wait(s_stop, (uint32_t)(np / flush - 1) & 1u, polls)) { ok = false; break; }
           tc_fence_after();
           store(flushed, false);
@@ -1334,8 +1337,19 @@ void launch_reduce(const float* part, int P, int n, float* out, int map, int K, 
       part, P, n, out, map, K, bpart, bout);
 }
 
+// Planes between two flushes of the weight gradient's accumulators: half of a
+// run of `tiles` tiles, at most 64 planes (512 additions).  A run without a
+// flush is further from 64 bits than tiles taken in turns over the cube are
+// (1.87e-6 against 1.76e-6 for 31x120x100, 1.44e-7 against 1.18e-7 for
+// 7x33x41: ragged tiles add less, and contiguous runs take the full ones
+// together), half a run is nearer for every size tried (6.7e-7 and 8.4e-8).  A
+// flush holds the MMAs up for 2.3 us: 31x120x100 64 -> 71 us, 7x33x41 22 -> 32,
+// 64x256x256 453 -> 477 (2.8e-5 -> 6.8e-6).
+int wgrad_flush(int tiles) { return tiles < 4 ? 1 : tiles < 128 ? tiles / 2 : 64; }
+
 // Weight (and, with bpart, bias) gradients of a 32 -> 32 layer: per-CTA partial
 // sums, one CTA per SM, at most part_slots(d) of them; returns their number.
+// flush: planes between two flushes, 0 for the rule above.
 int launch_wgrad_part(const bf16* a, const bf16* dz, float* part, float* bpart, const Dims& d, int flush, int sms,
                       cudaStream_t st) {
   int tx, ty;
@@ -1343,7 +1357,8 @@ int launch_wgrad_part(const bf16* a, const bf16* dz, float* part, float* bpart, 
   int P = part_slots(d);
   if (P > sms) P = sms;
   if (P > ntiles) P = ntiles;
-  k_wgrad_tc05<<<P, 288, wgrad05_smem(flush > 0), st>>>(a, dz, part, bpart, d, tx, ty, flush);
+  if (flush <= 0) flush = wgrad_flush(ntiles / P);
+  k_wgrad_tc05<<<P, 288, wgrad05_smem, st>>>(a, dz, part, bpart, d, tx, ty, flush);
   return P;
 }
 

@@ -175,3 +175,15 @@ def test_network_exact(netmod, shape, K):
     assert float(want.abs().max()) > 0 and torch.equal(g, want)
     net.close()
     assert netmod.wait_timeouts() == 0
+
+
+def test_weight_gradient_of_one_sign(netmod):
+    """The tensor core truncates every addition (one unit in the last place of the accumulator at most).  Over the 512
+    additions between two flushes, of terms of one size and sign, that is at most sum_i 2^-23 i / 512 = 256 * 2^-23 of
+    their sum; 215 tiles a block without a flush lose 8e-5."""
+    shape = (64, 256, 256)
+    g = torch.Generator(device="cuda").manual_seed(9)
+    a, dz = ((1 + torch.rand(shape + (32,), device="cuda", generator=g)).bfloat16() for _ in range(2))
+    dw, _ = conv_weights(a.double(), dz.double())
+    got, _ = netmod.conv3d_backward_weights(a, dz)
+    assert float(((got.double() - dw).abs() / dw).max()) <= 256 * 2.0 ** -23
