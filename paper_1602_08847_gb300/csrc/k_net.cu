@@ -6,7 +6,7 @@
 //
 // Feature maps are [nz][ny][nx][32] bfloat16 (64 bytes per voxel).  The
 // tensor-core kernels (below) march tiles of 1 x 16 x 8 voxels along the
-// channel axis.  The CUDA-core kernels of the 1 -> 32 layer work on output tiles
+// channel axis.  The CUDA-core kernels of the first and last layers work on output tiles
 // of 2 x 8 x 16 voxels (channel, row, column) whose scalar inputs, with a
 // one-voxel halo (4 x 10 x 18, zero outside the cube: the zero padding of the
 // layers), are staged in shared memory.
@@ -22,10 +22,9 @@
 //                 (M = (row offset, ci), N = (channel offset, co), K = voxels), tcgen05.mma
 //                 with the accumulators resident in tensor memory for the CTA's whole run.
 // The last layer's forward (prediction, or the loss and its gradient d6) is
-// the forward kernel with 16 columns an output (weights of maps K .. 15 zero);
-// its gradients are the 32 -> 32 kernels on d6 split into bfloat16 parts
-// (split3).  The 1 -> 32 layer (27 multiply-adds per voxel and output) runs on
-// the CUDA cores.  Every reduction over voxels is a per-block partial sum
+// the forward kernel with 16 columns an output (weights of maps K .. 15 zero).
+// Its gradients, whose operand d6 is float32, and the 1 -> 32 layer (27
+// multiply-adds per voxel and output) run on the CUDA cores.  Every reduction over voxels is a per-block partial sum
 // followed by a fixed-order sum: results do not depend on scheduling.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
@@ -151,29 +150,11 @@ struct LastArgs {
   const float* s;             // input scale (device scalar)
   const float* tx;            // EPI_LOSS: target cube [V]
   const bf16* taux;           // EPI_LOSS: target fields [nz][K-1][ny][nx]
-  bf16* d6;                   // EPI_LOSS: loss gradient [V][32], split in three (split3)
+  float* d6;                  // EPI_LOSS: loss gradient [V][K]
   double* lpart;              // EPI_LOSS: per-CTA partial sums [grid][K+1]
   float* out_x;               // EPI_PRED: cube [V]
   float* out_aux;             // EPI_PRED: fields [nz][K-1][ny][nx]
 };
-
-// The loss gradient of the last layer is float32.  It goes to the tensor cores
-// as three bfloat16 values that add up to it exactly, hi + mid + lo (8 bits of
-// its significand each), in a map of 32 features: map k's parts in features k,
-// 8 + k and 16 + k.  Its products with bfloat16 weights and maps are exact in
-// float32, so the two gradients of the last layer are the 32 -> 32 kernels.
-constexpr int kSplit = 8;                    // features between the parts
-__device__ __forceinline__ void split3(float v, float& hi, float& mid, float& lo) {
-  hi = __uint_as_float(__float_as_uint(v) & 0xffff0000u);
-  mid = lo = 0.f;
-  if (!(fabsf(v) <= 3.402823466e38f)) {      // infinity or NaN
-    hi = v;
-    return;
-  }
-  const float r = v - hi;
-  mid = __uint_as_float(__float_as_uint(r) & 0xffff0000u);
-  lo = r - mid;
-}
 
 // Sum of floats in two floats (Knuth's two-sum), for the few terms between two
 // additions to a double: double arithmetic runs at 1/64 of the float rate.
@@ -578,14 +559,13 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
             const int K = la.K;
             const size_t v = vox(d, z, y, x);
             const size_t a0 = ((size_t)z * (K > 1 ? K - 1 : 1)) * plane + (size_t)y * d.nx + x;
-            float part[EPI == EPI_LOSS ? 3 * kSplit : 1] = {};
 #pragma unroll
             for (int k = 0; k < kMaxOut; ++k) {
               if (k < K) {
                 const float zk = __uint_as_float(r[k]) + bn[k];
                 if constexpr (EPI == EPI_LOSS) {
                   const float rk = zk - (k == 0 ? tk[0] * inv_sc : tk[k]), lk = la.lam.v[k];
-                  split3(gk[k] * rk, part[k], part[kSplit + k], part[2 * kSplit + k]);
+                  la.d6[v * K + k] = gk[k] * rk;
                   // lam r^2 and r with their rounding errors where those are float32 values, else in double
                   const float p = lk * rk, q = p * rk;
                   if (q >= 1e-28f && q <= 1e30f) psum[0].add(q, fmaf(p, rk, -q) + fmaf(lk, rk, -p) * rk);
@@ -597,12 +577,6 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
                   else la.out_aux[a0 + (size_t)(k - 1) * plane] = fminf(fmaxf(zk, -1.f), 1.f);
                 }
               }
-            }
-            if constexpr (EPI == EPI_LOSS) {
-              uint4* o = reinterpret_cast<uint4*>(la.d6 + v * C);
-#pragma unroll
-              for (int q = 0; q < 3; ++q) o[q] = pack8(part + 8 * q);
-              o[3] = make_uint4(0u, 0u, 0u, 0u);
             }
           }
           if (EPI == EPI_LOSS && (no & 7) == 7) flush();
@@ -671,7 +645,6 @@ constexpr int WG_SUM = 3 * 3 * C * 96 * 4;              // flushed sums, 110592 
 constexpr int wgrad05_smem = WG_BAR + 256 + 128 + WG_SUM;
 static_assert(wgrad05_smem + 4096 <= muffin::kMaxDynSmem, "weight gradient shared memory");
 constexpr int WG_N = 3 * C;
-constexpr int kLastFlush = 4;                          // planes between two flushes, last layer
 // D f32, A/B bf16, both MN-major, N = n, M = 128
 __host__ __device__ constexpr uint32_t idesc_wgrad(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(n >> 3) << 17) |
@@ -983,6 +956,174 @@ k_first_fwd(const bf16* __restrict__ a0, const float* __restrict__ w, const floa
   }
 }
 
+// Gradients of the last layer.  Their sums are float32 multiply-adds rounded to
+// nearest, which the tensor cores do not offer: as 32 -> 32 gradients of d6 split
+// into three bfloat16 parts, exact products and all, they took 0.23 and 0.57 ms
+// instead of the times below, but truncated additions left the weight gradient 3
+// to 14 times further from 64 bits (31x120x100, five maps: 3.8e-8 -> 3.9e-7) and
+// the input gradient with a bias of 1e-6.
+
+// Two float32 multiply-adds in one instruction, each rounded to nearest.
+__device__ __forceinline__ void fma2(float2& acc, float2 a, float2 b) {
+  unsigned long long* c = reinterpret_cast<unsigned long long*>(&acc);
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(*c) : "l"(*reinterpret_cast<unsigned long long*>(&a)),
+      "l"(*reinterpret_cast<unsigned long long*>(&b)));
+}
+
+// g5[p][ci] = (a5[p][ci] > 0) * sum_tap sum_k d6[p - d(tap)][k] w[tap][k][ci].
+// A thread takes 16 of the features of four voxels (both channels of rows ty and
+// ty + 4), so that four 16-byte weight reads, the same for the whole warp, feed
+// 64 multiply-adds, and issues them in pairs; d6 lies in planes of one map, whose
+// lanes' reads are consecutive.  64x256x256, six maps: 1.58 ms (32 features of one
+// voxel a thread, d6 interleaved) -> 1.06, half of the FP32 rate; 1.21 without pairs.
+constexpr int LV = TZ * 2;            // voxels of a thread
+constexpr int kLastThreads = TV / LV * 2;
+template <int K>
+__global__ void __launch_bounds__(kLastThreads)
+k_last_bwd_data(const float* __restrict__ d6, const float* __restrict__ w, const bf16* __restrict__ a5,
+                bf16* __restrict__ g5, Dims d) {
+  extern __shared__ __align__(16) float smf[];
+  float* s_w = smf;                      // [27][K][32]
+  float* s_h = smf + NTAP * K * C;       // [K][HV]
+  for (int i = threadIdx.x; i < NTAP * K * C; i += blockDim.x) s_w[i] = w[i];
+  const int c0 = threadIdx.x / (TV / LV) * 16, tx = threadIdx.x % TX, ty = threadIdx.x % (TV / LV) / TX;
+  for (int tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) {
+    int z0, y0, x0;
+    tile_origin(tile, d, z0, y0, x0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < HV * K; i += blockDim.x) {
+      const int h = i / K, k = i - h * K;
+      const int hx = h % HX, r = h / HX, hy = r % HY, hz = r / HY;
+      const int gz = z0 - 1 + hz, gy = y0 - 1 + hy, gx = x0 - 1 + hx;
+      s_h[k * HV + h] = inside(d, gz, gy, gx) ? d6[vox(d, gz, gy, gx) * K + k] : 0.f;
+    }
+    __syncthreads();
+    float2 acc[LV][8];                   // voxel v: channel v / 2, row ty + 4 (v % 2)
+#pragma unroll
+    for (int v = 0; v < LV; ++v)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) acc[v][c] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int t = 0; t < NTAP; ++t) {
+      const int kz = t / 9, ky = (t / 3) % 3, kx = t % 3;
+      const float* h = s_h + ((2 - kz) * HY + ty + 2 - ky) * HX + tx + 2 - kx;
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        float2 dv[LV];
+#pragma unroll
+        for (int v = 0; v < LV; ++v) dv[v].x = dv[v].y = h[k * HV + (v / 2 * HY + v % 2 * 4) * HX];
+        const float4* wr = reinterpret_cast<const float4*>(s_w + (t * K + k) * C + c0);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float4 wv = wr[q];
+#pragma unroll
+          for (int v = 0; v < LV; ++v) {
+            fma2(acc[v][2 * q], dv[v], make_float2(wv.x, wv.y));
+            fma2(acc[v][2 * q + 1], dv[v], make_float2(wv.z, wv.w));
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < LV; ++v) {
+      const int z = z0 + v / 2, y = y0 + ty + v % 2 * 4, x = x0 + tx;
+      if (!inside(d, z, y, x)) continue;
+      const size_t at = vox(d, z, y, x) * C + c0;
+      const uint4* m = reinterpret_cast<const uint4*>(a5 + at);
+      uint4* o = reinterpret_cast<uint4*>(g5 + at);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        float mf[8], r[8];
+        unpack8(m[q], mf);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) r[e] = !(mf[e] > 0.f) ? 0.f : e & 1 ? acc[v][4 * q + e / 2].y : acc[v][4 * q + e / 2].x;
+        o[q] = pack8(r);
+      }
+    }
+  }
+}
+
+// part[b][tap][ci][k] = sum_p d6[p][k] a5[p + d(tap)][ci].  288 threads: thread
+// (kz, ky, ci) keeps the three taps kx = 0..2 of its row offset for all K maps in
+// registers and walks each tile row along x with a sliding window of three a5
+// values, so that one a5 read and the voxel's d6 values (one or two 16-byte reads,
+// the same for the whole block) feed 3 K multiply-adds.  64x256x256, six maps:
+// 1.55 ms (a 4-byte read for each d6 value, swizzled a5 rows) -> 1.32; two features
+// a thread 1.36, with pairs of multiply-adds 1.52.
+template <int K> __host__ __device__ constexpr int last_pitch() { return K == 1 ? 1 : K == 2 ? 2 : K <= 4 ? 4 : 8; }
+template <int K>
+__global__ void __launch_bounds__(288)
+k_wgrad_last(const float* __restrict__ d6, const bf16* __restrict__ a5, float* __restrict__ part, Dims d) {
+  constexpr int KP = last_pitch<K>();
+  extern __shared__ __align__(128) unsigned char smem[];     // a5 halo [HV][32] bfloat16, then d6 [TV][KP]
+  const uint32_t sa = smem_u32(smem);
+  float* s_d = reinterpret_cast<float*>(smem + HV * ROWB);
+  const int ci = threadIdx.x & 31, kzy = threadIdx.x >> 5, kz = kzy / 3, ky = kzy % 3;
+  const bf16* s_a = reinterpret_cast<const bf16*>(smem) + ci;
+  float acc[3][K];
+#pragma unroll
+  for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+    for (int k = 0; k < K; ++k) acc[kx][k] = 0.f;
+  for (int tile = blockIdx.x; tile < d.ntiles; tile += gridDim.x) {
+    int z0, y0, x0;
+    tile_origin(tile, d, z0, y0, x0);
+    __syncthreads();
+    for (int i = threadIdx.x; i < HV * 4; i += blockDim.x) {
+      const int c = i & 3, h = i >> 2;
+      const int hx = h % HX, t = h / HX, hy = t % HY, hz = t / HY;
+      const int gz = z0 - 1 + hz, gy = y0 - 1 + hy, gx = x0 - 1 + hx;
+      const bool ok = inside(d, gz, gy, gx);
+      cp_async16(sa + h * ROWB + c * 16, ok ? a5 + vox(d, gz, gy, gx) * C + c * 8 : a5, ok ? 16 : 0);
+    }
+    for (int i = threadIdx.x; i < TV * K; i += blockDim.x) {
+      const int r = i / K, k = i - r * K;
+      const int gz = z0 + (r >> 7), gy = y0 + ((r >> 4) & 7), gx = x0 + (r & 15);
+      s_d[r * KP + k] = inside(d, gz, gy, gx) ? d6[vox(d, gz, gy, gx) * K + k] : 0.f;
+    }
+    cp_async_wait_all();
+    __syncthreads();
+#pragma unroll 1
+    for (int row = 0; row < TZ * TY; ++row) {
+      const int tz = row >> 3, ty = row & 7;
+      const bf16* ar = s_a + ((tz + kz) * HY + ty + ky) * HX * C;   // halo row of this thread's taps
+      const float* dr = s_d + row * TX * KP;
+      float w0 = __bfloat162float(ar[0]), w1 = __bfloat162float(ar[C]);
+#pragma unroll 4
+      for (int tx = 0; tx < TX; ++tx) {
+        const float w2 = __bfloat162float(ar[(tx + 2) * C]);
+        float g[KP];
+        if constexpr (KP >= 4) {
+#pragma unroll
+          for (int q = 0; q < KP / 4; ++q) {
+            const float4 v = *reinterpret_cast<const float4*>(dr + tx * KP + 4 * q);
+            g[4 * q] = v.x; g[4 * q + 1] = v.y; g[4 * q + 2] = v.z; g[4 * q + 3] = v.w;
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < KP; ++k) g[k] = dr[tx * KP + k];
+        }
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          acc[0][k] = fmaf(g[k], w0, acc[0][k]);
+          acc[1][k] = fmaf(g[k], w1, acc[1][k]);
+          acc[2][k] = fmaf(g[k], w2, acc[2][k]);
+        }
+        w0 = w1;
+        w1 = w2;
+      }
+    }
+  }
+#pragma unroll
+  for (int kx = 0; kx < 3; ++kx) {
+    float* pp = part + ((size_t)blockIdx.x * (NTAP * C) + (kz * 9 + ky * 3 + kx) * C + ci) * K;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      pp[k] = acc[kx][k];
+    }
+  }
+}
+
 // part[b][tap][co] = sum_p g1[p][co] a0[p + d(tap)]; bpart[b][co] = sum_p g1[p][co].
 // Lane = co; each of the eight warps takes two tile rows of sixteen voxels and
 // keeps all 27 taps in registers: four voxels' g1 values and, row offset by row
@@ -1090,8 +1231,7 @@ constexpr int kReduceThreads = 64;
 // out[map(i)] = sum_b part[b*n + i] (fixed order, double accumulation), and with bout the C biases
 // bout[c] = sum_b bpart[b*C + c].
 // MAP_MID: i = (tap*32 + co)*32 + ci -> (co*32 + ci)*27 + tap; MAP_FIRST:
-// i = tap*32 + co -> co*27 + tap; MAP_LAST: i = (tap*K + k)*32 + ci -> (k*32 + ci)*27 + tap, the sum over the three
-// parts of the split loss gradient (features k, 8 + k, 16 + k of a 32 -> 32 weight gradient).
+// i = tap*32 + co -> co*27 + tap; MAP_LAST: i = (tap*32 + ci)*K + k -> (k*32 + ci)*27 + tap.
 __global__ void __launch_bounds__(kReduceThreads)
 k_reduce_part(const float* __restrict__ part, int P, int n, float* __restrict__ out, int map, int K,
               const float* __restrict__ bpart, float* __restrict__ bout) {
@@ -1101,16 +1241,11 @@ k_reduce_part(const float* __restrict__ part, int P, int n, float* __restrict__ 
     return;
   }
   int j = i;
-  double s;
+  const double s = sum_parts(part + i, P, n);
   if (map == MAP_LAST) {
-    const int ci = i & 31, r = i >> 5, k = r % K, t = r / K;
-    const float* p = part + (t * C + k) * C + ci;
-    s = sum_parts(p, P, WMID) + sum_parts(p + kSplit * C, P, WMID) + sum_parts(p + 2 * kSplit * C, P, WMID);
+    const int k = i % K, r = i / K, ci = r & 31, t = r >> 5;
     j = (k * C + ci) * NTAP + t;
-  } else {
-    s = sum_parts(part + i, P, n);
-  }
-  if (map == MAP_MID) {
+  } else if (map == MAP_MID) {
     const int t = i >> 10, co = (i >> 5) & 31, ci = i & 31;
     j = (co * C + ci) * NTAP + t;
   } else if (map == MAP_FIRST) {
@@ -1182,7 +1317,7 @@ struct KernelWeights {
   bf16* wf;     // [4][27][32 co][32 ci]   forward operands of layers 2..5
   bf16* wb;     // [4][27][32 ci][32 co]   flipped, transposed: input gradients
   float* bm;    // [4][32]
-  bf16* w6b;    // [27 flipped][32 ci][32]  last layer, input gradient: features k, 8 + k, 16 + k all the weight of map k
+  float* w6b;   // [27][K][32 ci]  last layer, input gradient; bfloat16 values
   bf16* w6t;    // [27][16 co][32 ci]  last layer, tcgen05 operand (rows K .. 15 zero)
   float* b6;    // [K]
 };
@@ -1218,9 +1353,8 @@ __global__ void k_unpack_params(const float* __restrict__ theta, KernelWeights k
   j -= 4 * LM;
   if (j < K * NTAP * C) {
     const int k = j / (C * NTAP), rem = j % (C * NTAP), ci = rem / NTAP, t = rem % NTAP;
-    const bf16 q = __float2bfloat16_rn(v);
-    for (int p = 0; p < 3; ++p) kw.w6b[((NTAP - 1 - t) * C + ci) * C + p * kSplit + k] = q;
-    kw.w6t[(t * kLastN + k) * C + ci] = q;
+    kw.w6b[(t * K + k) * C + ci] = round_bf16(v);
+    kw.w6t[(t * kLastN + k) * C + ci] = __float2bfloat16_rn(v);
   } else {
     kw.b6[j - K * NTAP * C] = v;
   }
@@ -1286,6 +1420,21 @@ int sm_count() {
   return n;
 }
 
+template <int K> constexpr int last_bwd_smem() { return K * (NTAP * C + HV) * 4; }
+template <int K> constexpr int wgrad_last_smem() { return HV * ROWB + TV * last_pitch<K>() * 4; }
+
+#define MNET_SWITCH_K(K, CALL) \
+  switch (K) {                 \
+    case 1: CALL(1); break;    \
+    case 2: CALL(2); break;    \
+    case 3: CALL(3); break;    \
+    case 4: CALL(4); break;    \
+    case 5: CALL(5); break;    \
+    case 6: CALL(6); break;    \
+    case 7: CALL(7); break;    \
+    default: CALL(8); break;   \
+  }
+
 cudaError_t configure_once() {
   static const cudaError_t err = [] {
     cudaError_t e;
@@ -1295,6 +1444,11 @@ cudaError_t configure_once() {
         (e = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_PRED>)) == cudaSuccess &&
         (e = muffin::allow_max_dyn_smem(k_conv_tc05<EPI_LOSS>)) == cudaSuccess)
       e = muffin::allow_max_dyn_smem(k_wgrad_tc05);
+#define CALL(KK)                                                                                       \
+  if (e == cudaSuccess && (e = muffin::allow_max_dyn_smem(k_last_bwd_data<KK>)) == cudaSuccess)        \
+  e = muffin::allow_max_dyn_smem(k_wgrad_last<KK>)
+    for (int K = 1; K <= kMaxOut; ++K) MNET_SWITCH_K(K, CALL)
+#undef CALL
     return e;
   }();
   return err;
@@ -1347,24 +1501,16 @@ void launch_reduce(const float* part, int P, int n, float* out, int map, int K, 
 // 64x256x256 453 -> 477 (2.8e-5 -> 6.8e-6).
 int wgrad_flush(int tiles) { return tiles < 4 ? 1 : tiles < 128 ? tiles / 2 : 64; }
 
-// Weight (and, with bpart, bias) gradients of a 32 -> 32 layer: per-CTA partial
-// sums, one CTA per SM, at most part_slots(d) of them; returns their number.
-// flush: planes between two flushes, 0 for the rule above.
-int launch_wgrad_part(const bf16* a, const bf16* dz, float* part, float* bpart, const Dims& d, int flush, int sms,
-                      cudaStream_t st) {
+// Weight and bias gradients of a 32 -> 32 layer: per-CTA partial sums (one CTA
+// per SM, at most part_slots(d) of them), then the fixed-order reduction.
+void launch_wgrad_mid(const bf16* a, const bf16* dz, float* part, float* bpart, float* dw, float* db, const Dims& d,
+                      int sms, cudaStream_t st) {
   int tx, ty;
   const int ntiles = tc05_tiles(d, tx, ty);
   int P = part_slots(d);
   if (P > sms) P = sms;
   if (P > ntiles) P = ntiles;
-  if (flush <= 0) flush = wgrad_flush(ntiles / P);
-  k_wgrad_tc05<<<P, 288, wgrad05_smem, st>>>(a, dz, part, bpart, d, tx, ty, flush);
-  return P;
-}
-
-void launch_wgrad_mid(const bf16* a, const bf16* dz, float* part, float* bpart, float* dw, float* db, const Dims& d,
-                      int sms, cudaStream_t st) {
-  const int P = launch_wgrad_part(a, dz, part, bpart, d, 0, sms, st);
+  k_wgrad_tc05<<<P, 288, wgrad05_smem, st>>>(a, dz, part, bpart, d, tx, ty, wgrad_flush(ntiles / P));
   launch_reduce(part, P, WMID, dw, MAP_MID, 1, bpart, db, st);
 }
 
@@ -1398,7 +1544,7 @@ struct muffin_net {
   bf16* act = nullptr;   // training: a1..a5; inference: two ping-pong maps
   bf16* gA = nullptr;
   bf16* gB = nullptr;
-  bf16* d6 = nullptr;    // loss gradient, split (split3)
+  float* d6 = nullptr;   // loss gradient [V][K]
 
   bf16* map(int i) const { return act + (size_t)i * d.nvox * C; }
 };
@@ -1425,7 +1571,7 @@ size_t net_layout(muffin_net* n, const Dims& d, int K, int training, char* base)
   kw.wf = (bf16*)take(4 * WMID * 2);
   kw.wb = (bf16*)take(4 * WMID * 2);
   kw.bm = (float*)take(4 * C * 4);
-  kw.w6b = (bf16*)take(WMID * 2);
+  kw.w6b = (float*)take(NTAP * K * C * 4);
   kw.w6t = (bf16*)take(NTAP * kLastN * C * 2);
   kw.b6 = (float*)take(K * 4);
   float* s = (float*)take(4);
@@ -1439,7 +1585,7 @@ size_t net_layout(muffin_net* n, const Dims& d, int K, int training, char* base)
   bf16* act = (bf16*)take((training ? 5 : 2) * V * C * 2);
   bf16* gA = (bf16*)take(training ? V * C * 2 : 0);
   bf16* gB = (bf16*)take(training ? V * C * 2 : 0);
-  bf16* d6 = (bf16*)take(training ? V * C * 2 : 0);
+  float* d6 = (float*)take(training ? V * K * 4 : 0);
   if (n) {
     n->theta = theta; n->mom1 = m1; n->mom2 = m2; n->grad = grad; n->kw = kw;
     n->s = s; n->mpart = mpart; n->lpart = lpart; n->loss = loss; n->part = part; n->bpart = bpart;
@@ -1495,24 +1641,28 @@ void last_predict(muffin_net* n, float* x, float* aux) {
   launch_tc05<EPI_PRED>(a5_of(n), n->kw.w6t, n->kw.b6, nullptr, nullptr, n->d, n->sms, n->st, la);
 }
 
-// Last layer of the training pass: loss, its gradient d6 (split),
-// the layer's weight and bias gradients, and the gradient of a5's
-// pre-activation into g5.
+// Last layer of the training pass: loss, its gradient d6, the layer's weight
+// and bias gradients, and the gradient of a5's pre-activation into g5.
 void last_train(muffin_net* n, const float* tx, const bf16* taux, bf16* g5) {
   const Dims& d = n->d;
-  bf16* d6 = n->d6;
   bf16* a5 = a5_of(n);
   LastArgs la = last_args(n);
   la.tx = tx;
   la.taux = taux;
-  la.d6 = d6;
+  la.d6 = n->d6;
   la.lpart = n->lpart;
   launch_tc05<EPI_LOSS>(a5, n->kw.w6t, n->kw.b6, nullptr, nullptr, d, n->sms, n->st, la);
   k_loss_final<<<1, n->K + 1, 0, n->st>>>(n->lpart, tc05_grid(d, n->sms), n->K, n->lam, d.nvox, n->loss,
                                           n->grad + b_offset(5, n->K));
-  const int P = launch_wgrad_part(a5, d6, n->part, nullptr, d, kLastFlush, n->sms, n->st);
-  launch_reduce(n->part, P, NTAP * n->K * C, n->grad + w_offset(5), MAP_LAST, n->K, nullptr, nullptr, n->st);
-  launch_conv(EPI_MASK, d6, n->kw.w6b, nullptr, a5, g5, d, n->sms, n->st);
+  int P = part_slots(d);
+  if (P > 2 * n->sms) P = 2 * n->sms;
+  const int grid = d.ntiles < 4 * n->sms ? d.ntiles : 4 * n->sms;
+#define CALL(KK)                                                                      \
+  k_wgrad_last<KK><<<P, 288, wgrad_last_smem<KK>(), n->st>>>(n->d6, a5, n->part, d);  \
+  k_last_bwd_data<KK><<<grid, kLastThreads, last_bwd_smem<KK>(), n->st>>>(n->d6, n->kw.w6b, a5, g5, d)
+  MNET_SWITCH_K(n->K, CALL)
+#undef CALL
+  launch_reduce(n->part, P, NTAP * C * n->K, n->grad + w_offset(5), MAP_LAST, n->K, nullptr, nullptr, n->st);
 }
 
 // Loss and gradient into n->grad (training contexts).
@@ -1538,7 +1688,6 @@ void loss_and_grad(muffin_net* n, const float* y, const float* tx, const bf16* t
 void unpack_params(muffin_net* n) {
   const int np = param_count(n->K);
   cudaMemsetAsync(n->kw.w6t, 0, NTAP * kLastN * C * 2, n->st);
-  cudaMemsetAsync(n->kw.w6b, 0, WMID * 2, n->st);
   k_unpack_params<<<(np + 255) / 256, 256, 0, n->st>>>(n->theta, n->kw, n->K);
 }
 

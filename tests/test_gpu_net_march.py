@@ -187,3 +187,73 @@ def test_weight_gradient_of_one_sign(netmod):
     dw, _ = conv_weights(a.double(), dz.double())
     got, _ = netmod.conv3d_backward_weights(a, dz)
     assert float(((got.double() - dw).abs() / dw).max()) <= 256 * 2.0 ** -23
+
+
+def bare_net(netmod, shape, K, b5, w6, lam):
+    """A training net whose weights are zero but for the last layer's: its feature map is max(b5, 0) at every voxel."""
+    theta = torch.zeros(netmod.n_params(K), dtype=torch.float64, device="cuda")
+    last = netmod.n_params(K) - K * (32 * 27 + 1)
+    theta[last - 32:last] = b5
+    theta[last:last + K * 32 * 27] = w6
+    return netmod.WarmStartNet(shape, training=True, theta=theta.float(), n_out=K, out_weight=lam), last
+
+
+@pytest.mark.parametrize("shape,K", [((31, 120, 100), 1), ((31, 120, 100), 6), ((64, 200, 136), 3), ((7, 33, 41), 8)])
+def test_last_weight_gradient_rounds_to_nearest(netmod, shape, K):
+    """Terms of one sign and of many exponents, so that truncated additions would show as a bias (4e-7 over 32 of them).
+    float32 sums rounded to nearest: a chain of n terms has an rms error of 0.289 2^-23 sqrt(n / 3) of its sum, P
+    independent ones a sqrt(P)-th of that; four times it, and the rounding of the result.  That holds for map 0, whose
+    targets are float32 values; the fields' are bfloat16, whose sums leave few different remainders."""
+    nz, ny, nx = shape
+    V = nz * ny * nx
+    b5 = 1 + (4 * torch.arange(32, device="cuda").double() + 1) / 128
+    net, last = bare_net(netmod, shape, K, b5, 0.0, [V / 2.0] * K)      # factor of the loss gradient: 1
+    g = torch.Generator(device="cuda").manual_seed(3)
+    y = torch.ones(shape, device="cuda")
+    tx = torch.exp2(-6 * torch.rand(shape, device="cuda", generator=g))
+    ta = torch.exp2(-6 * torch.rand((nz, K - 1, ny, nx), device="cuda", generator=g)).bfloat16() if K > 1 else None
+    _, grad = net.loss_grad(y, tx, ta)
+    d6 = -tx.double()[..., None] if ta is None else -torch.cat([tx[:, None].double(), ta.double()], 1).permute(0, 2, 3, 1)
+    dw, _ = conv_weights(b5.expand(*shape, 32), d6)
+    got = grad[last:last + K * 32 * 27].view(K, 32, 3, 3, 3).double()
+    tiles = ((nx + 15) // 16) * ((ny + 7) // 8) * ((nz + 1) // 2)
+    P = min(tiles, 304)
+    n = 256 * -(-tiles // P)
+    bound = 4 * 0.289 * 2.0 ** -23 * (n / 3 / P) ** 0.5 + 2.0 ** -24
+    err = ((got - dw) / dw)[0]
+    assert float(err.abs().max()) <= bound
+    assert abs(float(err.mean())) <= bound / 32 ** 0.5        # and no bias: the features' errors are independent
+    net.close()
+
+
+def test_last_input_gradient_rounds_to_nearest(netmod):
+    """One map, weights 1, a loss gradient of v everywhere: the last layer's input gradient is the sum of v over the
+    taps inside the cube.  v is chosen so that 27 additions rounded to nearest end two to four units above a tie of the
+    rounding to bfloat16, and truncated ones more than four below it.  Seen through the bias gradient of the layer
+    before, the sum of the map over the cube."""
+    import numpy as np
+
+    def chain(v, n, nearest):
+        s = np.zeros_like(v)
+        for _ in range(n):
+            exact = s.astype(np.float64) + v                  # exact in double
+            t = exact.astype(np.float32)
+            s = t if nearest else np.where(t > exact, np.nextafter(t, np.float32(0)), t)
+        return s
+
+    def above_tie(s):                                         # units of the last place above a tie of bfloat16
+        return (s.view(np.uint32) & 0xFFFF).astype(int) - 0x8000
+
+    vs = np.arange(0x3F800001, 0x40000000, 7, dtype=np.uint32).view(np.float32)
+    up, down = above_tie(chain(vs, 27, True)), above_tie(chain(vs, 27, False))
+    v = vs[(up >= 2) & (up <= 4) & (down < -4) & (down > -1000)][:1]
+    shape = (6, 40, 40)
+    V = 6 * 40 * 40
+    net, last = bare_net(netmod, shape, 1, 2.0 ** -100, 1.0, [V / 2.0])
+    _, grad = net.loss_grad(torch.ones(shape, device="cuda"), torch.full(shape, -float(v[0]), device="cuda"))
+    want = 0.0
+    for inner, count in ((4 * 38 * 38, 27), (2 * 38 * 38 + 2 * 4 * 38 * 2, 18), (2 * 38 * 4 + 4 * 4, 12), (2 * 4, 8)):
+        want += inner * float(torch.from_numpy(chain(v, count, True)).bfloat16()[0])
+    # a bfloat16 unit at the interior voxels is at least 2^-8 of most of the sum
+    assert abs(grad[last - 32:last].double() / want - 1).max() <= 1e-4
+    net.close()
