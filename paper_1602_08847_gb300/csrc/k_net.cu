@@ -350,18 +350,8 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
   Runs runs(tiles_x * tiles_y, d.nz);
   int col, za, zb;
   bool ok = true;
-  // EPI_LOSS: sums of up to eight tiles (lam r^2, then r of each map), and per thread the doubles they go to
-  __shared__ double s_loss[EPI == EPI_LOSS ? (kMaxOut + 1) * 128 : 1];
-  double* tsum = s_loss + (EPI == EPI_LOSS ? threadIdx.x & 127 : 0);
-  Pair psum[EPI == EPI_LOSS ? kMaxOut + 1 : 1];
-  auto flush = [&] {
-#pragma unroll
-    for (int k = 0; k <= kMaxOut; ++k) {
-      if (k > la.K) break;
-      tsum[128 * k] += (double)psum[k].hi + (double)psum[k].lo;
-      psum[k] = Pair{0.f, 0.f};
-    }
-  };
+  // EPI_LOSS: sums of lam r^2 and of r of each map
+  double l2 = 0.0, lsum[EPI == EPI_LOSS ? kMaxOut : 1] = {};
 
   if (warp >= 4 && warp < 8) {
     // ---------------- loaders: planes za-1 .. zb of each stretch, two planes in flight behind the newest
@@ -476,11 +466,6 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
     if constexpr (EPI == EPI_LOSS) {
 #pragma unroll
       for (int k = 0; k < kMaxOut; ++k) gk[k] = (float)(2.0 / (double)d.nvox * la.lam.v[k]);
-#pragma unroll
-      for (int k = 0; k <= kMaxOut; ++k) {
-        tsum[128 * k] = 0.0;
-        psum[k] = Pair{0.f, 0.f};
-      }
     }
     const size_t plane = (size_t)d.ny * d.nx;
     const int m = warp * 32 + lane;
@@ -564,14 +549,10 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
               if (k < K) {
                 const float zk = __uint_as_float(r[k]) + bn[k];
                 if constexpr (EPI == EPI_LOSS) {
-                  const float rk = zk - (k == 0 ? tk[0] * inv_sc : tk[k]), lk = la.lam.v[k];
+                  const float rk = zk - (k == 0 ? tk[0] * inv_sc : tk[k]);
                   la.d6[v * K + k] = gk[k] * rk;
-                  // lam r^2 and r with their rounding errors where those are float32 values, else in double
-                  const float p = lk * rk, q = p * rk;
-                  if (q >= 1e-28f && q <= 1e30f) psum[0].add(q, fmaf(p, rk, -q) + fmaf(lk, rk, -p) * rk);
-                  else tsum[0] += (double)lk * rk * rk;
-                  if (fabsf(rk) <= 1e30f) psum[k + 1].add(rk, 0.f);
-                  else tsum[128 * (k + 1)] += rk;
+                  l2 += (double)la.lam.v[k] * rk * rk;
+                  lsum[k] += rk;
                 } else {
                   if (k == 0) la.out_x[v] = fmaxf(sc * zk, 0.f);
                   else la.out_aux[a0 + (size_t)(k - 1) * plane] = fminf(fmaxf(zk, -1.f), 1.f);
@@ -579,11 +560,9 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
               }
             }
           }
-          if (EPI == EPI_LOSS && (no & 7) == 7) flush();
         }
       }
     }
-    if (EPI == EPI_LOSS) flush();
   }
   const bool fin = mbar_drain(s_fin, 0);   // every copy and MMA issued, also after a give-up: TMEM is freed below
   tc_fence_before();
@@ -593,10 +572,14 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
   if constexpr (EPI == EPI_LOSS) {
     // lpart[block] = (sum_k lam_k sum_p r_k^2, sum_p r_0, ..., sum_p r_{K-1}), fixed order
-    for (int k = 0; k <= la.K; ++k) {
-      const double t = muffin::block_sum(threadIdx.x < 128 ? tsum[128 * k] : 0.0, s_red);
-      if (threadIdx.x == 0) la.lpart[(size_t)blockIdx.x * (la.K + 1) + k] = t;
+    const double t2 = muffin::block_sum(l2, s_red);
+    if (threadIdx.x == 0) la.lpart[(size_t)blockIdx.x * (la.K + 1)] = t2;
+#pragma unroll
+    for (int k = 0; k < kMaxOut; ++k) {
+      if (k >= la.K) break;
       __syncthreads();
+      const double t = muffin::block_sum(lsum[k], s_red);
+      if (threadIdx.x == 0) la.lpart[(size_t)blockIdx.x * (la.K + 1) + 1 + k] = t;
     }
   }
 }

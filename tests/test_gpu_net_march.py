@@ -257,3 +257,44 @@ def test_last_input_gradient_rounds_to_nearest(netmod):
     # a bfloat16 unit at the interior voxels is at least 2^-8 of most of the sum
     assert abs(grad[last - 32:last].double() / want - 1).max() <= 1e-4
     net.close()
+
+
+def test_loss_sums_keep_the_bits_of_doubles(netmod):
+    """Residuals that are integers at the voxels of four columns along the channel axis, where one thread sums a
+    stretch of them, and zero elsewhere: one large value in eight and small odd ones behind it, which a sum in float
+    pairs cannot hold.  The sums of lam r^2, and of r, stay below 2^53, so doubles hold every partial sum; those of r
+    cancel to a small integer."""
+    shape = (64, 200, 136)
+    V = 64 * 200 * 136
+    y = torch.ones(shape, device="cuda")
+    g = torch.Generator().manual_seed(11)
+    columns = [(5, 7), (77, 30), (150, 99), (199, 135)]
+    lam = 2 ** 18 - 1
+    net, last = bare_net(netmod, shape, 1, 0.0, 0.0, [float(lam)])
+    tx = torch.zeros(shape)
+    for r, c in columns:
+        v = 2 * torch.randint(2, 5, (64,), generator=g) + 1                  # lam r^2 of 23 to 25 bits
+        v[::8] = 2 * torch.randint(10000, 11000, (8,), generator=g) + 1      # of 47
+        tx[:, r, c] = -v.float()
+    total = lam * int((tx.double() ** 2).sum())
+    loss, _ = net.loss_grad(y, tx.cuda())
+    assert total < 2 ** 53 and loss == total / V
+    net.close()
+    net, last = bare_net(netmod, shape, 1, 0.0, 0.0, [1.0])
+    for small in (3, -1001):
+        tx = torch.zeros(shape)
+        for r, c in columns:
+            v = 2 * torch.randint(2 ** 22, 2 ** 23, (56,), generator=g) + 1  # odd, 24 bits
+            v[::8] <<= 23
+            v = v.tolist()
+            rest = small - sum(v)                          # in three floats of at most 24 bits
+            for _ in range(3):
+                step = max(abs(rest).bit_length() - 24, 0)
+                part = (abs(rest) >> step << step) * (1 if rest > 0 else -1)
+                v.append(part)
+                rest -= part
+            assert rest == 0
+            tx[:len(v), r, c] = -torch.tensor(v, dtype=torch.float64).float()
+        _, grad = net.loss_grad(y, tx.cuda())
+        assert float(grad[-1]) == float(torch.tensor(2.0 * len(columns) * small / V, dtype=torch.float64).float())
+    net.close()
