@@ -36,6 +36,7 @@
 #include <string>
 
 #include "device.cuh"
+#include "exact_sum.cuh"
 #include "muffin.h"
 #include "muffin_net.h"
 
@@ -154,17 +155,6 @@ struct LastArgs {
   double* lpart;              // EPI_LOSS: per-CTA partial sums [grid][K+1]
   float* out_x;               // EPI_PRED: cube [V]
   float* out_aux;             // EPI_PRED: fields [nz][K-1][ny][nx]
-};
-
-// Sum of floats in two floats (Knuth's two-sum), for the few terms between two
-// additions to a double: double arithmetic runs at 1/64 of the float rate.
-struct Pair {
-  float hi, lo;
-  __device__ __forceinline__ void add(float x, float e) {
-    const float t = hi + x, b = t - hi;
-    lo += ((hi - (t - b)) + (x - b)) + e;
-    hi = t;
-  }
 };
 
 // ------------------------------------------------------------------ 32 -> 32 layers on tcgen05 (UMMA), marching along z
@@ -1186,8 +1176,9 @@ enum { MAP_MID = 1, MAP_FIRST = 2, MAP_LAST = 3 };
 // sum_b p[b * n], b = 0 .. P-1, eight at a time in flight: the loop is one load
 // latency per trip (a 31x120x100 layer's weight gradient took 99.7 us with four
 // loads a trip and blocks of 256, 79.5 so, in blocks of 64 and with the biases
-// in the same launch).  The eight are added as a float pair, then to the double
-// (with a conversion and an addition in FP64 for each the call takes 79.5 us, so 72.1).
+// in the same launch).  The eight are added in three floats (Sum3), then to the
+// double, which holds what a double addition for each would: 152 partial sums of 27648
+// outputs take 12.5 us so, 20.7 with one each (float pairs, 11.2, lost bits).
 __device__ __forceinline__ double sum_parts(const float* __restrict__ p, int P, size_t n) {
   double s = 0.0;
   int b = 0;
@@ -1195,11 +1186,11 @@ __device__ __forceinline__ double sum_parts(const float* __restrict__ p, int P, 
     float v[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[e] = p[(size_t)(b + e) * n];
-    Pair t{0.f, 0.f};
+    muffin::Sum3 t;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) t.add(v[e], 0.f);
-    if (fabsf(t.hi) <= 1e37f && fabsf(t.lo) <= 1e37f) {
-      s += (double)t.hi + (double)t.lo;
+    for (int e = 0; e < 8; ++e) t.add(v[e]);
+    if (fabsf(t.hi) <= 1e37f && fabsf(t.mid) <= 1e37f) {
+      t.into(s);
     } else {                         // infinities, NaN, or sums near the end of the range
 #pragma unroll 1
       for (int e = 0; e < 8; ++e) s += p[(size_t)(b + e) * n];

@@ -93,3 +93,39 @@ def test_scale_rounds_the_double_product(lib, offset):
             want = (x.double() * f).float()
             same = (got.view(torch.int32) == want.view(torch.int32)) | (got.isnan() & want.isnan())
             assert bool(same.all()), (f, x[~same][:3], got[~same][:3], want[~same][:3])
+
+
+def cancelling(g, groups, small):
+    """8 * groups + 3 integers of at most 24 significant bits, one large in eight and small odd ones behind it, that add
+    up to `small`; every partial sum is below 2^53."""
+    v = 2 * torch.randint(2 ** 22, 2 ** 23, (8 * groups,), generator=g) + 1
+    v[::8] <<= 23
+    v = v.tolist()
+    rest = small - sum(v)
+    for _ in range(3):
+        step = max(abs(rest).bit_length() - 24, 0)
+        v.append((abs(rest) >> step << step) * (1 if rest > 0 else -1))
+        rest -= v[-1]
+    assert rest == 0
+    return v
+
+
+@pytest.mark.parametrize("groups", [1, 2, 5, 19])
+def test_reduction_of_partial_sums_keeps_the_bits_of_doubles(lib, groups):
+    """Weight and bias gradients from their blocks' partial sums (k_net.cu), through mnet::launch_reduce."""
+    f = lib.lib._ZN4mnet13launch_reduceEPKfiiPfiiS1_S2_P11CUstream_st
+    f.argtypes, f.restype = [_P, ctypes.c_int, ctypes.c_int, _P, ctypes.c_int, ctypes.c_int, _P, _P, _P], None
+    g = torch.Generator().manual_seed(groups)
+    n, P, want = 64, 8 * groups + 3, list(range(-48, 48))
+    v = torch.tensor([cancelling(g, groups, s) for s in want], dtype=torch.float64).T.contiguous()     # [P][n + 32]
+    assert torch.equal(v.float().double(), v)
+    part, bpart = v[:, :n].float().cuda(), v[:, n:].float().cuda()
+    out, bout = torch.zeros(27 * 1024, device="cuda"), torch.zeros(32, device="cuda")
+    for bad in (None, float("inf"), float("nan")):
+        if bad is not None:
+            part[1, 5] = bad
+            want[5] = bad
+        f(part.contiguous().data_ptr(), P, n, out.data_ptr(), 1, 1, bpart.contiguous().data_ptr(), bout.data_ptr(), stream())
+        # output i = (tap 0, co i / 32, ci i % 32) goes to (co 32 + ci) 27
+        got = torch.cat([out[:27 * n:27], bout]).cpu()
+        assert torch.equal(torch.nan_to_num(got, nan=1e30), torch.nan_to_num(torch.tensor(want, dtype=torch.float32), nan=1e30))
