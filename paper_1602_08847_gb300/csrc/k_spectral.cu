@@ -345,13 +345,18 @@ int spectral_take_timeouts() {
 //   c[2i]   = sum_{l < M} C[2i][l] s[l]      (M = ceil(L/2); s of the middle of an odd L is x)
 //   c[2i+1] = sum_{l < H} C[2i+1][l] d[l]    (H = floor(L/2))
 // and back, e[l] = sum_i C[2i][l] y[2i], o[l] = sum_i C[2i+1][l] y[2i+1],
-// T[l] = e[l] + o[l], T[L-1-l] = e[l] - o[l]: half the multiply-adds.  The
-// products are register tiled: a thread holds 8 rows x 4 pixels, one 16-byte
+// T[l] = e[l] + o[l], T[L-1-l] = e[l] - o[l]: half the multiply-adds.  The even
+// coefficients of smooth spectra are small differences of sums that are now of
+// twice the size, and came out 1.4 times further from 64 bits than the plain
+// product's; the rows of C but the first add up to zero, so a value near the mean
+// of s is taken from it first (fold_mean; the first row keeps s): nearer than the
+// plain product from about 20 channels on.  With fewer the rounding of s itself
+// shows, and up to kPlainSum channels the analysis takes them in turn.
+// The products are register tiled: a thread holds 8 rows x 4 pixels, one 16-byte
 // shared-memory read and two uniform table reads feed 32 multiply-adds, so the
 // FP32 pipe bounds the larger L and DRAM the smaller ones.  (One row a thread,
 // as the norm still does it, reads two values for every multiply-add.)
-// 256x256x96: 332 -> 95 us per launch; 256x256x200: 1560 -> 280; 1024x1024x7:
-// 81 -> 41.
+// 256x256x96: 332 -> 102 us per launch; 256x256x200: 1560 -> 323.
 struct FoldDims {
   int M, H, KE, KO;   // even and odd rows, and both rounded up to 8
 };
@@ -390,7 +395,10 @@ void spectral_fold_tables(int L, float* out) {
   }
 }
 
+// acc[r] += sign tab[r] x
+template <int SIGN = 1>
 __device__ __forceinline__ void fold_row(float4 (&acc)[8], const float* __restrict__ tab, float4 x) {
+  if (SIGN < 0) x = make_float4(-x.x, -x.y, -x.z, -x.w);
   const float4 a = __ldg(reinterpret_cast<const float4*>(tab)), b = __ldg(reinterpret_cast<const float4*>(tab) + 1);
   const float w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
@@ -402,9 +410,24 @@ __device__ __forceinline__ void fold_row(float4 (&acc)[8], const float* __restri
   }
 }
 
+// About the mean over l of s: of up to eight of its H rows (x: row 0, tp floats a
+// row), zero where that is no ordinary number.  Whatever it is, the sums with it
+// taken off are the same but for their rounding.
+__device__ __forceinline__ float4 fold_mean(const float* x, int H, int tp) {
+  const int n = H < 8 ? H : 8;
+  float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int i = 0; i < n; ++i) {
+    const float4 s = *reinterpret_cast<const float4*>(x + (2 * i + 1) * H / (2 * n) * tp);
+    m = make_float4(m.x + s.x, m.y + s.y, m.z + s.z, m.w + s.w);
+  }
+  const float w = 1.0f / n;
+  auto ordinary = [](float v) { return fabsf(v) <= 1e30f ? v : 0.f; };
+  return make_float4(ordinary(w * m.x), ordinary(w * m.y), ordinary(w * m.z), ordinary(w * m.w));
+}
+
 // LPR lanes cover the 4 LPR pixels of a subtile; S subtiles a block; a unit of
 // LPR threads takes 8 rows of one subtile at a time.  npix is a multiple of 4 LPR.
-template <int LPR, int MODE>
+template <int LPR, int MODE, bool PAIRS>
 __global__ void __launch_bounds__(256, 2)
 k_spectral_fold(SpecArgs a, int npix, int L, int S) {
   extern __shared__ __align__(16) float sm[];
@@ -412,7 +435,7 @@ k_spectral_fold(SpecArgs a, int npix, int L, int S) {
   const FoldDims f = fold_dims(L);
   const int tp = SUB * S, p0 = blockIdx.x * tp;
   const int np = npix - p0 < tp ? npix - p0 : tp;       // pixels of this block
-  float* X = sm;                  // [L][tp]: s[l] in row l, d[l] in row L-1-l
+  float* X = sm;                  // [L][tp]: s[l] in row l, d[l] in row L-1-l; up to kPlainSum channels x[l]
   float* Y = sm + (size_t)L * tp; // [L][tp]: the new duals
   const size_t P = (size_t)npix;
   const float *E = a.fold, *Et = E + (size_t)f.M * f.KE, *O = Et + (size_t)f.M * f.KE, *Ot = O + (size_t)f.H * f.KO;
@@ -424,14 +447,17 @@ k_spectral_fold(SpecArgs a, int npix, int L, int S) {
     for (int i = threadIdx.x; i < f.M * nch; i += blockDim.x) {
       const int l = i / nch, c = 4 * (i % nch);
       if (c >= np) continue;
-      const float4 u = __ldcg(reinterpret_cast<const float4*>(D + (size_t)l * P + c));
+      float4 u = __ldcg(reinterpret_cast<const float4*>(D + (size_t)l * P + c));
       if (l < f.H) {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(D + (size_t)(L - 1 - l) * P + c));
-        *reinterpret_cast<float4*>(X + l * tp + c) = make_float4(u.x + v.x, u.y + v.y, u.z + v.z, u.w + v.w);
-        *reinterpret_cast<float4*>(X + (L - 1 - l) * tp + c) = make_float4(u.x - v.x, u.y - v.y, u.z - v.z, u.w - v.w);
-      } else {
-        *reinterpret_cast<float4*>(X + l * tp + c) = u;
+        float4 v = __ldcg(reinterpret_cast<const float4*>(D + (size_t)(L - 1 - l) * P + c));
+        if (PAIRS) {
+          const float4 w = v;
+          v = make_float4(u.x - w.x, u.y - w.y, u.z - w.z, u.w - w.w);
+          u = make_float4(u.x + w.x, u.y + w.y, u.z + w.z, u.w + w.w);
+        }
+        *reinterpret_cast<float4*>(X + (L - 1 - l) * tp + c) = v;
       }
+      *reinterpret_cast<float4*>(X + l * tp + c) = u;
     }
     __syncthreads();
     const int ge = f.KE / 8, go = f.KO / 8;
@@ -446,11 +472,43 @@ k_spectral_fold(SpecArgs a, int npix, int L, int S) {
         vo[r] = acc[r];
         if (r0 + r < nr) vo[r] = __ldcg(reinterpret_cast<const float4*>(a.V + (size_t)(2 * (r0 + r) + odd) * P + p0 + px));
       }
-      const float* x = X + px + (odd ? (size_t)(L - 1) * tp : 0);
-      const int step = odd ? -tp : tp;
+      const float* x = X + px;
+      const float* y = x + (size_t)(L - 1) * tp;          // y - l tp: row L - 1 - l
       const float* tab = (odd ? O : E) + r0;
+      auto at = [](const float* q) { return *reinterpret_cast<const float4*>(q); };
+      if constexpr (PAIRS) {
+        if (odd) {
 #pragma unroll 4
-      for (int l = 0; l < nr; ++l) fold_row(acc, tab + (size_t)l * K, *reinterpret_cast<const float4*>(x + l * step));
+          for (int l = 0; l < f.H; ++l) fold_row(acc, tab + (size_t)l * K, at(y - l * tp));
+        } else {
+          const float4 m = fold_mean(x, f.H, tp);
+#pragma unroll 4
+          for (int l = 0; l < f.H; ++l) {
+            const float4 s = at(x + l * tp);
+            fold_row(acc, tab + (size_t)l * K, make_float4(s.x - m.x, s.y - m.y, s.z - m.z, s.w - m.w));
+          }
+          if (f.M > f.H) {
+            const float4 s = at(x + f.H * tp);
+            fold_row(acc, tab + (size_t)f.H * K, make_float4(s.x - 0.5f * m.x, s.y - 0.5f * m.y, s.z - 0.5f * m.z, s.w - 0.5f * m.w));
+          }
+          if (r0 == 0) {                 // c[0]: all of the sum
+            float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int l = 0; l < f.M; ++l) {
+              const float4 s = at(x + l * tp);
+              const float w = __ldg(tab + (size_t)l * K);
+              c = make_float4(fmaf(w, s.x, c.x), fmaf(w, s.y, c.y), fmaf(w, s.z, c.z), fmaf(w, s.w, c.w));
+            }
+            acc[0] = c;
+          }
+        }
+      } else {
+        for (int l = 0; l < nr; ++l) fold_row(acc, tab + (size_t)l * K, at(x + l * tp));
+        if (odd) {
+          for (int l = f.H - 1; l >= 0; --l) fold_row<-1>(acc, tab + (size_t)l * K, at(y - l * tp));
+        } else {
+          for (int l = f.H - 1; l >= 0; --l) fold_row(acc, tab + (size_t)l * K, at(y - l * tp));
+        }
+      }
 #pragma unroll
       for (int r = 0; r < 8; ++r) {
         if (r0 + r >= nr) continue;
@@ -492,6 +550,13 @@ k_spectral_fold(SpecArgs a, int npix, int L, int S) {
   }
 }
 
+// Channels up to which the analysis sums one by one.  Error of the even
+// coefficients of smooth spectra, plain product / pairs with the mean taken off
+// (modelled on the host): 6 channels 1.1e-8 / 4.7e-8, 12 3.0e-8 / 4.7e-8, 21
+// 6.8e-8 / 4.5e-8, 200 1.3e-7 / 4.7e-8.  Time of the spectral step in a pass,
+// pairs / one by one: 1024x1024x8 75 / 77 us, 512x512x12 17.2 / 18.2, 128x128x37
+// 18.2 / 20.7, 256x256x96 102 / 124.
+constexpr int kPlainSum = 16;
 template <int LPR> static cudaError_t spec_fold(const SpecArgs& a, int npix, int L, int mode, cudaStream_t s) {
   constexpr int SUB = 4 * LPR;
   const int groups = fold_dims(L).KE / 8;
@@ -502,8 +567,9 @@ template <int LPR> static cudaError_t spec_fold(const SpecArgs& a, int npix, int
   int warps = (groups * S * LPR + 31) / 32;
   warps = warps < 1 ? 1 : warps > 8 ? 8 : warps;
   const int grid = (npix + SUB * S - 1) / (SUB * S);
-  if (mode == SPEC_UPDATE) k_spectral_fold<LPR, SPEC_UPDATE><<<grid, 32 * warps, smem(S), s>>>(a, npix, L, S);
-  else k_spectral_fold<LPR, SPEC_TONLY><<<grid, 32 * warps, smem(S), s>>>(a, npix, L, S);
+  if (mode == SPEC_TONLY) k_spectral_fold<LPR, SPEC_TONLY, true><<<grid, 32 * warps, smem(S), s>>>(a, npix, L, S);
+  else if (LPR == 8 || L > kPlainSum) k_spectral_fold<LPR, SPEC_UPDATE, true><<<grid, 32 * warps, smem(S), s>>>(a, npix, L, S);
+  else if constexpr (LPR == 16) k_spectral_fold<LPR, SPEC_UPDATE, false><<<grid, 32 * warps, smem(S), s>>>(a, npix, L, S);
   return cudaGetLastError();
 }
 
@@ -667,10 +733,11 @@ cudaError_t spectral_configure(int L) {
     return cudaErrorInvalidValue;
   }
   cudaError_t e;
-  if ((e = allow_max_dyn_smem(k_spectral_fold<16, SPEC_UPDATE>))) return e;
-  if ((e = allow_max_dyn_smem(k_spectral_fold<16, SPEC_TONLY>))) return e;
-  if ((e = allow_max_dyn_smem(k_spectral_fold<8, SPEC_UPDATE>))) return e;
-  if ((e = allow_max_dyn_smem(k_spectral_fold<8, SPEC_TONLY>))) return e;
+  if ((e = allow_max_dyn_smem(k_spectral_fold<16, SPEC_UPDATE, true>))) return e;
+  if ((e = allow_max_dyn_smem(k_spectral_fold<16, SPEC_UPDATE, false>))) return e;
+  if ((e = allow_max_dyn_smem(k_spectral_fold<16, SPEC_TONLY, true>))) return e;
+  if ((e = allow_max_dyn_smem(k_spectral_fold<8, SPEC_UPDATE, true>))) return e;
+  if ((e = allow_max_dyn_smem(k_spectral_fold<8, SPEC_TONLY, true>))) return e;
   if ((e = allow_max_dyn_smem(k_spectral_dense<SPEC_UPDATE>))) return e;
   if ((e = allow_max_dyn_smem(k_spectral_dense<SPEC_NORM>))) return e;
   return allow_max_dyn_smem(k_spectral_dense<SPEC_TONLY>);
