@@ -202,6 +202,19 @@ cudaError_t launch_permute_planes(const float* src, float* dst, int n, int L, in
                                   cudaStream_t s);
 cudaError_t launch_nonfinite_count(const float* x, size_t n, int* count, cudaStream_t s);
 
+// SMs of the device (152 where there is none to ask).
+inline int device_sms() {
+  static const int sms = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaGetLastError();
+      return 152;
+    }
+    return v;
+  }();
+  return sms;
+}
+
 // How far ahead in launch order a block prefetches inputs into L2: the blocks
 // of kernel fn resident on the device at once (one wave), times
 // MUFFIN_L2_PREFETCH when that is set (0: no prefetch; 2: two waves ahead).

@@ -406,18 +406,6 @@ k_fine_adjoint_m(int J, int L, const float* __restrict__ rin, size_t rin_stride,
 }  // namespace march
 
 // ------------------------------------------------------------------ host side
-static int sm_count() {
-  static const int sms = [] {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-      cudaGetLastError();
-      return 152;
-    }
-    return v;
-  }();
-  return sms;
-}
-
 // How a kernel's rows are split over blocks.  A step (one row of every
 // resident block) was measured to take about lat + warp * (warps on the SM)
 // microseconds; the cheapest in steps times step time wins.
@@ -429,7 +417,7 @@ constexpr StepTime kAnalysisStep[4] = {{}, {0.30f, 0.020f}, {0.38f, 0.024f}, {0.
 constexpr StepTime kAdjointStep[4] = {{}, {0.30f, 0.020f}, {0.33f, 0.030f}, {0.27f, 0.050f}};
 
 static Split split_rows(int n, int L, int lag, int minb, StepTime t, bool chunks) {
-  const int sms = sm_count();
+  const int sms = device_sms();
   auto steps = [&](int rows) { return (rows + lag + march::kUnroll - 1) / march::kUnroll * march::kUnroll + 2; };
   Split best{n, 1};
   float best_cost = 1e30f;

@@ -563,7 +563,7 @@ template <int LPR> static cudaError_t spec_fold(const SpecArgs& a, int npix, int
   auto smem = [&](int S) { return (size_t)2 * L * SUB * S * sizeof(float); };
   // subtiles: at least four warps of work in a block, while two or three blocks fit an SM; no fewer blocks than SMs
   int S = 1;
-  while (groups * S * LPR / 32 < 4 && smem(2 * S) <= 72 * 1024 && npix / (SUB * 2 * S) >= 152) S *= 2;
+  while (groups * S * LPR / 32 < 4 && smem(2 * S) <= 72 * 1024 && npix / (SUB * 2 * S) >= device_sms()) S *= 2;
   int warps = (groups * S * LPR + 31) / 32;
   warps = warps < 1 ? 1 : warps > 8 ? 8 : warps;
   const int grid = (npix + SUB * S - 1) / (SUB * S);
