@@ -42,7 +42,10 @@ using vec::st4;
 using vec::sub4;
 
 constexpr int kCoarseWarps = 4;     // warps of a block (independent of one another)
-constexpr int kAheadCoarse = 4;     // rows between a row's L2 prefetch and its use
+// Rows between a row's L2 prefetch and its use.  1024x1024x64, two levels / one
+// level, us per launch in a pass: 587 / 415 at 1 row, 493 / 378 at 2, 485 / 374 at
+// 3, 487 / 375 at 4, 491 / 390 at 6, 509 / 386 at 8.
+constexpr int kAheadCoarse = 4;
 constexpr int M = 128;              // side of a sub-image
 
 template <int NL> struct CoarseM {
@@ -241,7 +244,11 @@ k_coarse_m(int n, int J, int j1, int units, const float* c_in, float* r_out, flo
 }  // namespace march
 
 // One or two levels on 128 x 128 sub-images at the largest split (N = 1024),
-// 512 of them at least (above).  Smaller images reach 64 x 64 sub-images and
+// 512 of them (8 channels) at least.  Pass of 1024 x 1024 x L with one level, us,
+// block kernel / march: L = 4 197 / 213, 5 254 / 246, 6 276 / 308, 7 300 / 326, 8
+// 352 / 332, 9 381 / 395, 10 431 / 423, 12 514 / 489, 16 625 / 564; with two: 4 230
+// / 262, 5 301 / 289, 6 324 / 368, 7 352 / 385, 8 414 / 402, 9 450 / 452, 10 511 /
+// 481, 12 605 / 543, 16 743 / 621.  Smaller images reach 64 x 64 sub-images and
 // their resident kernel with a larger split; at 512 x 512 x 64, J = 4, the
 // march at j1 = 2 is the faster wavelet half on its own (0.240 against 0.283
 // ms), but hides less of the spectral step beside it (pass 0.515 against 0.483).
