@@ -108,7 +108,6 @@ bool daubechies_lowpass(int p, double* h) {
 
 constexpr float kUnionScale = 0.35355339059327373f;   // 1/sqrt(8)
 constexpr int kRowsPerBlock = 8;
-constexpr int kColRun = 4;
 constexpr int kMinTile = 32;      // smallest level of the row-group kernels
 
 // The kernels below run one body per basis, instantiated for its filter length
@@ -322,29 +321,25 @@ k_idwt_group_sum(const float* __restrict__ U, const float* __restrict__ llin, fl
   put16(S + l * P + (size_t)(blockIdx.x * R + row) * n + 16 * run, acc, kUnionScale);
 }
 
-// ------------------------------------------------------------------ small levels
+// ------------------------------------------------------------------ small levels, at most 16 x 16
 
-// Analysis of one whole level, rows and columns fused through shared memory.
-// A block owns a slab of SC consecutive columns k0 .. k0 + SC - 1 of the
-// row-transformed plane (all lo columns or all hi columns, H % SC == 0):
-// it computes them for all M rows into shared memory (row filter, inputs read
-// through L1), then filters each of its columns: the low-low quadrant feeds
-// the next level (written to `ll`, which the caller alternates between two
-// scratch planes so that no level overwrites the plane it reads), every final
-// coefficient updates U as in dwt_cols_body.  grid (M / SC, 1, 8 L), shared
-// memory M * SC floats.
+// Analysis of one whole level of at most 16 x 16, rows and columns fused through
+// shared memory.  A block owns the low or the high half of the columns of the
+// row-transformed plane: it computes them for all M rows into shared memory (row
+// filter, inputs read through L1), then filters each of its columns: the low-low
+// quadrant feeds the next level (written to `ll`, which the caller alternates
+// between two scratch planes so that no level overwrites the plane it reads),
+// every final coefficient updates U.  grid (2, 1, 8 L), shared memory M H floats.
 template <int MODE, int TAPS>
 __device__ __forceinline__ void dwt_level_body(const float* __restrict__ src0, const float* __restrict__ llin,
-                                               float* __restrict__ ll, float* __restrict__ U, int n, int M, int SC,
+                                               float* __restrict__ ll, float* __restrict__ U, int n, int M,
                                                int level0, int last, float kk, float rho, float* __restrict__ sY) {
   const int z = blockIdx.z, b = z & 7, l = z >> 3;
   const int H = M >> 1, m = M - 1;
   const size_t P = (size_t)n * n;
-  const int k0 = blockIdx.x * SC;
-  const bool hic = k0 >= H;                    // slab of high-pass (detail) columns
-  const int kb = hic ? k0 - H : k0;
+  const bool hic = blockIdx.x == 1;            // the high-pass (detail) columns
   const float* src = level0 ? src0 + (size_t)l * P : llin + (size_t)z * P;
-  const int lsc = __ffs(SC) - 1;
+  const int lsc = __ffs(H) - 1;
   // the basis' filters in registers (constant-memory reads per tap would cost an issue slot each)
   float hf[TAPS], gf[TAPS];
 #pragma unroll
@@ -352,10 +347,10 @@ __device__ __forceinline__ void dwt_level_body(const float* __restrict__ src0, c
     hf[t] = c_dbh[b][t];
     gf[t] = c_dbg[b][t];
   }
-  for (int idx = threadIdx.x; idx < M * SC; idx += blockDim.x) {
-    const int r = idx >> lsc, j = idx & (SC - 1);
+  for (int idx = threadIdx.x; idx < M * H; idx += blockDim.x) {
+    const int r = idx >> lsc, j = idx & (H - 1);
     const float* row = src + (size_t)r * n;
-    const int base = 2 * (kb + j);
+    const int base = 2 * j;
     // taps in aligned pairs: (2k + t) is even for even t and M is even, so x[t + 1] follows x[t]
     float x[TAPS];
 #pragma unroll
@@ -381,8 +376,8 @@ __device__ __forceinline__ void dwt_level_body(const float* __restrict__ src0, c
       *u = w;
     }
   };
-  for (int idx = threadIdx.x; idx < H * SC; idx += blockDim.x) {
-    const int q = idx >> lsc, j = idx & (SC - 1), c = k0 + j;
+  for (int idx = threadIdx.x; idx < H * H; idx += blockDim.x) {
+    const int q = idx >> lsc, j = idx & (H - 1), c = hic ? H + j : j;
     float x[TAPS];
 #pragma unroll
     for (int t = 0; t < TAPS; ++t) x[t] = sY[(((2 * q + t) & m) << lsc) + j];
@@ -399,11 +394,11 @@ __device__ __forceinline__ void dwt_level_body(const float* __restrict__ src0, c
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(128)
 k_dwt_level(const float* __restrict__ src0, const float* __restrict__ llin, float* __restrict__ ll,
-            float* __restrict__ U, int n, int M, int SC, int level0, int last, float kk, float rho) {
+            float* __restrict__ U, int n, int M, int level0, int last, float kk, float rho) {
   extern __shared__ float sY[];
-#define CALL(T) dwt_level_body<MODE, T>(src0, llin, ll, U, n, M, SC, level0, last, kk, rho, sY)
+#define CALL(T) dwt_level_body<MODE, T>(src0, llin, ll, U, n, M, level0, last, kk, rho, sY)
   MUFFIN_DB_DISPATCH(CALL)
 #undef CALL
 }
@@ -415,7 +410,7 @@ template <int TAPS>
 __device__ __forceinline__ void idwt_cols_body(const float* __restrict__ U, const float* __restrict__ W2,
                                                float* __restrict__ W1, int n, int M, int coarsest) {
   const int z = blockIdx.z, b = z & 7;
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  const int c = threadIdx.x;
   const int H = M >> 1, m = M - 1;
   if (c >= M) return;
   const size_t P = (size_t)n * n;
@@ -430,9 +425,7 @@ __device__ __forceinline__ void idwt_cols_body(const float* __restrict__ U, cons
     ge[s2] = c_dbg[b][par + 2 * s2];
   }
 #pragma unroll 1
-  for (int j = 0; j < kColRun; ++j) {
-    const int i = (blockIdx.y * kColRun + j) * blockDim.y + threadIdx.y;
-    if (i >= M) break;
+  for (int i = threadIdx.y; i < M; i += blockDim.y) {
     float a[TAPS / 2], d[TAPS / 2];
 #pragma unroll
     for (int s2 = 0; s2 < TAPS / 2; ++s2) {
@@ -583,14 +576,6 @@ cudaError_t dwt_configure() {
 
 // ------------------------------------------------------------------ launchers
 
-// Columns per slab of the fused analysis: at most 32, at most 8192 / M (32 KB
-// of shared memory), at most H.
-static int dwt_slab(int M) {
-  int sc = 32;
-  while (sc > 1 && (sc > M / 2 || sc * M > 8192)) sc >>= 1;
-  return sc;
-}
-
 template <int MODE>
 static void dwt_level(const Geom& g, const DwtArgs& a, int j, cudaStream_t s) {
   const int n = g.n, Z = kDbBases * g.L, M = n >> j, last = j == g.J - 1;
@@ -604,9 +589,8 @@ static void dwt_level(const Geom& g, const DwtArgs& a, int j, cudaStream_t s) {
     k_dwt_rows<MODE, Q><<<dim3(M / 2 / Q, 1, Z), M < 512 ? M : 512, (size_t)(2 * Q + kMaxTaps - 2) * M * sizeof(float), s>>>(
         a.src, llin, ll, a.U, n, M, j == 0, last, kk, rho);
   } else {
-    const int sc = dwt_slab(M);
-    k_dwt_level<MODE><<<dim3(M / sc, 1, Z), 256, (size_t)M * sc * sizeof(float), s>>>(a.src, llin, ll, a.U, n, M, sc,
-                                                                                  j == 0, last, kk, rho);
+    k_dwt_level<MODE><<<dim3(2, 1, Z), 128, (size_t)M * (M / 2) * sizeof(float), s>>>(
+        a.src, llin, ll, a.U, n, M, j == 0, last, kk, rho);
   }
 }
 
@@ -634,10 +618,9 @@ cudaError_t launch_dwt_adjoint(const Geom& g, const DwtArgs& a, cudaStream_t s) 
       continue;
     }
     // small levels come first and hand their images on in W2
-    k_idwt_cols<<<dim3((M + 31) / 32, (M + 8 * kColRun - 1) / (8 * kColRun), Z), dim3(32, 8), 0, s>>>(
-        a.U, a.W2, a.W1, n, M, coarsest);
-    if (j > 0) k_idwt_rows<<<dim3(1, (M + kRowsPerBlock - 1) / kRowsPerBlock, Z), 128, 0, s>>>(a.W1, a.W2, n, M);
-    else k_idwt_rows_sum<<<dim3(1, (M + kRowsPerBlock - 1) / kRowsPerBlock, g.L), 256, 0, s>>>(a.W1, a.S, n);
+    k_idwt_cols<<<dim3(1, 1, Z), dim3(32, 8), 0, s>>>(a.U, a.W2, a.W1, n, M, coarsest);
+    if (j > 0) k_idwt_rows<<<dim3(1, (M + kRowsPerBlock - 1) / kRowsPerBlock, Z), 64, 0, s>>>(a.W1, a.W2, n, M);
+    else k_idwt_rows_sum<<<dim3(1, (M + kRowsPerBlock - 1) / kRowsPerBlock, g.L), 64, 0, s>>>(a.W1, a.S, n);
   }
   return cudaGetLastError();
 }

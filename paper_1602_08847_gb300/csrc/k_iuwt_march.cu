@@ -22,7 +22,8 @@
 // Measured at 512 x 512 x 256, three fine levels (us per launch, tiles before,
 // march now, bytes each must move): analysis 490 -> 362 (2.15 GB: 5.9 TB/s, DRAM
 // bound), adjoint 670 -> 286 (1.34 GB: 4.7 TB/s; 12 warps per SM, bound by the
-// latency and the issue slots of a step).  256 x 256 x 64, two levels: 28.7 ->
+// latency and the issue slots of a step; three levels spill 36 bytes a thread at
+// 168 registers for N below 1024).  256 x 256 x 64, two levels: 28.7 ->
 // 22.8 and 40.9 -> 21.0.
 
 #include "internal.h"

@@ -494,29 +494,29 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
           if (inside(d, z, y, x)) {
             const size_t base = vox(d, z, y, x) * C;
             float v[C];
-    #pragma unroll
+#pragma unroll
             for (int c = 0; c < C; ++c) v[c] = __uint_as_float(r[c]);
             if (EPI == EPI_MASK) {
               if (mask) {
                 const uint4* mp = reinterpret_cast<const uint4*>(mask + base);
-    #pragma unroll
+#pragma unroll
                 for (int q = 0; q < 4; ++q) {
                   float mf[8];
                   unpack8(mp[q], mf);
-    #pragma unroll
+#pragma unroll
                   for (int e = 0; e < 8; ++e)
                     if (!(mf[e] > 0.f)) v[8 * q + e] = 0.f;
                 }
               }
             } else {
-    #pragma unroll
+#pragma unroll
               for (int c = 0; c < C; ++c) {
                 v[c] += bn[c];
                 if (EPI == EPI_RELU) v[c] = fmaxf(v[c], 0.f);
               }
             }
             uint4* o = reinterpret_cast<uint4*>(out + base);
-    #pragma unroll
+#pragma unroll
             for (int q = 0; q < 4; ++q) o[q] = pack8(v + 8 * q);
           }
         } else {
@@ -530,7 +530,7 @@ k_conv_tc05(const bf16* __restrict__ in, const bf16* __restrict__ wk, const floa
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           tc_fence_before();
           mbar_arrive(s_read + 8 * acc);
-            if (inside(d, z, y, x)) {
+          if (inside(d, z, y, x)) {
             const int K = la.K;
             const size_t v = vox(d, z, y, x);
             const size_t a0 = ((size_t)z * (K > 1 ? K - 1 : 1)) * plane + (size_t)y * d.nx + x;

@@ -555,7 +555,7 @@ k_spectral_fold(SpecArgs a, int npix, int L, int S) {
 // (modelled on the host): 6 channels 1.1e-8 / 4.7e-8, 12 3.0e-8 / 4.7e-8, 21
 // 6.8e-8 / 4.5e-8, 200 1.3e-7 / 4.7e-8.  Time of the spectral step in a pass,
 // pairs / one by one: 1024x1024x8 75 / 77 us, 512x512x12 17.2 / 18.2, 128x128x37
-// 18.2 / 20.7, 256x256x96 102 / 124.
+// 18.2 / 20.7, 256x256x96 102 / 124.  (One by one spills 4 bytes a thread.)
 constexpr int kPlainSum = 16;
 template <int LPR> static cudaError_t spec_fold(const SpecArgs& a, int npix, int L, int mode, cudaStream_t s) {
   constexpr int SUB = 4 * LPR;
