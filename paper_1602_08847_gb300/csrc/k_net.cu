@@ -1465,15 +1465,21 @@ void launch_reduce(const float* part, int P, int n, float* out, int map, int K, 
       part, P, n, out, map, K, bpart, bout);
 }
 
-// Planes between two flushes of the weight gradient's accumulators: half of a
-// run of `tiles` tiles, at most 64 planes (512 additions).  A run without a
-// flush is further from 64 bits than tiles taken in turns over the cube are
-// (1.87e-6 against 1.76e-6 for 31x120x100, 1.44e-7 against 1.18e-7 for
-// 7x33x41: ragged tiles add less, and contiguous runs take the full ones
-// together), half a run is nearer for every size tried (6.7e-7 and 8.4e-8).  A
-// flush holds the MMAs up for 2.3 us: 31x120x100 64 -> 71 us, 7x33x41 22 -> 32,
-// 64x256x256 453 -> 477 (2.8e-5 -> 6.8e-6).
-int wgrad_flush(int tiles) { return tiles < 4 ? 1 : tiles < 128 ? tiles / 2 : 64; }
+// Planes between two flushes of the weight gradient's accumulators, for runs of
+// `tiles` tiles.  A run without a flush is further from 64 bits than tiles taken
+// in turns over the cube are, because ragged tiles add less and contiguous runs
+// take the full ones together (31x120x100 1.87e-6 against 1.76e-6, 7x33x41 1.44e-7
+// against 1.18e-7, 64x256x256 2.85e-5 against 2.75e-5).  So half a run where more
+// than a tenth of the tiles' voxels lies outside the cube, else fifteen sixteenths,
+// which is enough (1.33e-6, 8.4e-8, 2.39e-5) and moves the sums of long runs by
+// less than 1e-5.  A flush holds the MMAs up for 2.3 us: kernel of 31x120x100 64
+// -> 66 us, 7x33x41 22 -> 32, 64x256x256 453 -> 456.
+int wgrad_flush(const Dims& d, int ntiles, int P) {
+  const int tiles = ntiles / P;
+  const bool ragged = 10 * d.nvox < 9LL * ntiles * U_TY * U_TX;
+  const int f = ragged ? tiles / 2 : tiles * 15 / 16;
+  return f < 1 ? 1 : f;
+}
 
 // Weight and bias gradients of a 32 -> 32 layer: per-CTA partial sums (one CTA
 // per SM, at most part_slots(d) of them), then the fixed-order reduction.
@@ -1484,7 +1490,7 @@ void launch_wgrad_mid(const bf16* a, const bf16* dz, float* part, float* bpart, 
   int P = part_slots(d);
   if (P > sms) P = sms;
   if (P > ntiles) P = ntiles;
-  k_wgrad_tc05<<<P, 288, wgrad05_smem, st>>>(a, dz, part, bpart, d, tx, ty, wgrad_flush(ntiles / P));
+  k_wgrad_tc05<<<P, 288, wgrad05_smem, st>>>(a, dz, part, bpart, d, tx, ty, wgrad_flush(d, ntiles, P));
   launch_reduce(part, P, WMID, dw, MAP_MID, 1, bpart, db, st);
 }
 
