@@ -1473,7 +1473,7 @@ void launch_reduce(const float* part, int P, int n, float* out, int map, int K, 
 // than a tenth of the tiles' voxels lies outside the cube, else fifteen sixteenths,
 // which is enough (1.33e-6, 8.4e-8, 2.39e-5) and moves the sums of long runs by
 // less than 1e-5.  A flush holds the MMAs up for 2.3 us: kernel of 31x120x100 64
-// -> 66 us, 7x33x41 22 -> 32, 64x256x256 453 -> 456.
+// -> 66 us, 7x33x41 22 -> 32, 64x256x256 453 -> 468.
 int wgrad_flush(const Dims& d, int ntiles, int P) {
   const int tiles = ntiles / P;
   const bool ragged = 10 * d.nvox < 9LL * ntiles * U_TY * U_TX;
